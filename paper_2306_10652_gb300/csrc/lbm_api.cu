@@ -432,7 +432,7 @@ int ensure_allocated(lbm_problem *p)
             p->st[k].rhi = dev_alloc(p, np * sizeof(float));
             p->st[k].rlo = (float *)dev_alloc(p, np * sizeof(float));
             if (!p->st[k].g || !p->st[k].rhi || !p->st[k].rlo) return LBM_ENOMEM;
-            // the partner of an odd last component stays empty (k_init writes it, set_state does not)
+            // the partner of an odd last component is empty (k_init and k_from_f64 write st[0]'s)
             if (np > nf && (cudaMemsetAsync(p->st[k].g, 0, np * (p->Q - 1) * sizeof(float), p->stream) != cudaSuccess ||
                             cudaMemsetAsync(p->st[k].rhi, 0, np * sizeof(float), p->stream) != cudaSuccess ||
                             cudaMemsetAsync(p->st[k].rlo, 0, np * sizeof(float), p->stream) != cudaSuccess))

@@ -526,6 +526,14 @@ __global__ void k_from_f64(const Params P, const double *__restrict__ in, StateB
                 st.rlo[st.at(i, N, r)] = (float)(rho - (double)hi);
             }
         }
+        // the empty partner of an odd last component: what the state held before may
+        // not be finite, and the passes sum over both components of a pair
+        if (sizeof(S) == 4 && (NC & 1) && st.paired) {
+#pragma unroll
+            for (int k = 0; k < NS; ++k) g[st.at(NC, k, NS, N, r)] = (S)0;
+            st.rhi_f()[st.at(NC, N, r)] = 0.0f;
+            st.rlo[st.at(NC, N, r)] = 0.0f;
+        }
     }
 }
 
