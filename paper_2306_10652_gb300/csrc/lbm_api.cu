@@ -63,10 +63,8 @@ struct lbm_problem {
     // kGraphSteps steps, for longer runs (by starting buffer; the number is even)
     cudaGraphExec_t chunk_exec[2] = {nullptr, nullptr};
     long long chunk_launches = 0;
-    bool no_graph = false;         // the stream cannot be captured
-    // lbm_step may capture: on a stream that orders itself with the legacy stream a
-    // capture would fail other threads' calls to the latter
-    bool quiet_capture = false;
+    bool no_graph = false;         // the steps could not be captured: not tried again
+    cudaStream_t cap = nullptr;    // where steps are captured: the handle's own stream, or one made for it
     long long launches = 0;
     KernelTimer *timer = nullptr;  // lbm_timing_enable: per-kernel CUDA-event timing (null: off)
     long long monitor_step = -1;
@@ -376,15 +374,10 @@ int ensure_allocated(lbm_problem *p)
     if (!p->stream) {
         if (p->opt.stream) {
             p->stream = (cudaStream_t)p->opt.stream;
-            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-            unsigned int flags = 0;
-            p->quiet_capture = cudaStreamIsCapturing(p->stream, &cs) == cudaSuccess &&
-                               cs == cudaStreamCaptureStatusNone &&
-                               cudaStreamGetFlags(p->stream, &flags) == cudaSuccess && (flags & cudaStreamNonBlocking);
         } else {
             if (cudaStreamCreateWithFlags(&p->stream, cudaStreamNonBlocking) != cudaSuccess)
                 return LBM_ECUDA;
-            p->own_stream = p->quiet_capture = true;
+            p->own_stream = true;
         }
     }
     build_params(p);
@@ -704,8 +697,32 @@ int step_loop(lbm_problem *p, long long n);
 constexpr long long kGraphSteps = 16;
 constexpr long long kGraphNodes = 1LL << 22;  // components x nodes
 
+// Captures n steps from the current buffer into *exec; the state and the counters
+// stay as they are.  Returns 0 if the steps were captured.
+int capture_steps(lbm_problem *p, long long n, cudaGraphExec_t *exec, long long *launches)
+{
+    const long long steps0 = p->steps, launches0 = p->launches;
+    const int cur0 = p->cur;
+    cudaStream_t const user = p->stream;
+    if (p->own_stream) p->cap = p->stream;  // nobody else has it
+    const int st = capture_graph(
+        &p->cap,
+        [&](cudaStream_t s) {
+            p->stream = s;
+            return step_loop(p, n);
+        },
+        exec);
+    p->stream = user;
+    *launches = p->launches - launches0;
+    p->cur = cur0;
+    p->steps = steps0;
+    p->launches = launches0;
+    p->sticky = LBM_OK;
+    return st;
+}
+
 // Replays as many whole chunks of the n steps as there are; *done receives the
-// steps taken (0 if the stream cannot be captured).
+// steps taken (0 if the caller is capturing the stream or the steps cannot be captured).
 int run_chunks(lbm_problem *p, long long n, long long *done)
 {
     *done = 0;
@@ -717,36 +734,10 @@ int run_chunks(lbm_problem *p, long long n, long long *done)
         p->psi_valid = true;
     }
     const int c = p->cur;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(p->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return LBM_OK;  // the caller is capturing: launch by launch
-    }
-    if (!p->chunk_exec[c]) {
-        if (cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-            cudaGetLastError();
-            p->no_graph = true;
-            return LBM_OK;
-        }
-        const long long steps0 = p->steps, launches0 = p->launches;
-        const int st = step_loop(p, kGraphSteps);
-        cudaGraph_t g = nullptr;
-        const cudaError_t ce = cudaStreamEndCapture(p->stream, &g);
-        // the capture recorded the steps without running them: undo the bookkeeping
-        p->cur = c;
-        p->steps = steps0;
-        p->chunk_launches = p->launches - launches0;
-        p->launches = launches0;
-        p->sticky = LBM_OK;
-        cudaError_t ie = cudaErrorUnknown;
-        if (!st && ce == cudaSuccess && g) ie = cudaGraphInstantiate(&p->chunk_exec[c], g, 0);
-        if (g) cudaGraphDestroy(g);
-        if (ie != cudaSuccess) {
-            cudaGetLastError();
-            p->chunk_exec[c] = nullptr;
-            p->no_graph = true;
-            return LBM_OK;
-        }
+    if (being_captured(p->stream)) return LBM_OK;  // launch by launch
+    if (!p->chunk_exec[c] && capture_steps(p, kGraphSteps, &p->chunk_exec[c], &p->chunk_launches)) {
+        p->no_graph = true;
+        return LBM_OK;
     }
     for (; n - *done >= kGraphSteps; *done += kGraphSteps) {
         if (cudaGraphLaunch(p->chunk_exec[c], p->stream) != cudaSuccess) return p->sticky = LBM_ECUDA;
@@ -998,8 +989,7 @@ int lbm_step(lbm_problem *p, long long n)
     if (p->timer) p->timer->last_end = nullptr;  // other work may have been enqueued since
     if (p->resident) return resident_steps(p, n);
     // a few chunks at least, and steps short enough for their launches to matter
-    if (n >= 3 * kGraphSteps && every == 0 && !p->timer && (long long)p->nc * p->N <= kGraphNodes &&
-        p->quiet_capture) {
+    if (n >= 3 * kGraphSteps && every == 0 && !p->timer && (long long)p->nc * p->N <= kGraphNodes) {
         long long done = 0;
         const int st = run_chunks(p, n, &done);
         if (st) return st;
@@ -1026,6 +1016,7 @@ int lbm_step_graph(lbm_problem *p, long long n)
         p->launches += 1;
         p->psi_valid = true;
     }
+    if (being_captured(p->stream)) return step_loop(p, n);
     if (n >= 2 * kGraphSteps) {  // chunks, and what is left launch by launch
         long long done = 0;
         const int st = run_chunks(p, n, &done);
@@ -1040,33 +1031,7 @@ int lbm_step_graph(lbm_problem *p, long long n)
         p->graph_n = n;
     }
     const int c = p->cur;
-    if (!p->graph_exec[c]) {
-        const long long steps0 = p->steps, launches0 = p->launches;
-        cudaGraph_t g = nullptr;
-        if (cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-            cudaGetLastError();
-            return lbm_step(p, n);  // the stream cannot be captured (for example, already capturing)
-        }
-        const int st = step_loop(p, n);
-        const cudaError_t ce = cudaStreamEndCapture(p->stream, &g);
-        // the capture recorded the steps without running them: undo the bookkeeping
-        p->cur = c;
-        p->steps = steps0;
-        p->graph_launches = p->launches - launches0;
-        p->launches = launches0;
-        if (st || ce != cudaSuccess || !g) {
-            if (g) cudaGraphDestroy(g);
-            cudaGetLastError();
-            p->sticky = LBM_OK;
-            return st ? st : LBM_ECUDA;
-        }
-        const cudaError_t ie = cudaGraphInstantiate(&p->graph_exec[c], g, 0);
-        cudaGraphDestroy(g);
-        if (ie != cudaSuccess) {
-            p->graph_exec[c] = nullptr;
-            return LBM_ECUDA;
-        }
-    }
+    if (!p->graph_exec[c] && capture_steps(p, n, &p->graph_exec[c], &p->graph_launches)) return step_loop(p, n);
     if (cudaGraphLaunch(p->graph_exec[c], p->stream) != cudaSuccess) return p->sticky = LBM_ECUDA;
     p->launches += p->graph_launches;
     p->steps += n;
@@ -1368,6 +1333,7 @@ int lbm_destroy(lbm_problem *p)
         delete p->timer;
     }
     dev_free_all(p);
+    if (p->cap && !p->own_stream) cudaStreamDestroy(p->cap);
     if (p->own_stream && p->stream) cudaStreamDestroy(p->stream);
     delete p;
     return LBM_OK;

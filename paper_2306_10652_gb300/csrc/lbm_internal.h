@@ -61,6 +61,49 @@ inline void kt_end(KernelTimer *t, cudaStream_t s)
     if (t) t->end(s);
 }
 
+// Captures what record(stream) enqueues as a graph and instantiates it.  `own` is a
+// stream that nobody but the caller's object uses, created here if null: a capture
+// belongs to its stream, so on a stream of the user's the launches of other threads
+// (and of other handles) made meanwhile would go into this graph instead of running.
+// The nodes do not depend on the stream; the graph may be launched on any.  Relaxed
+// mode, for the stream and the thread: no call here touches a capture that another
+// thread has under way, and none of theirs ends this one.  Returns 0, or -1 with
+// *exec null if the work could not be captured.
+template <typename Record> int capture_graph(cudaStream_t *own, Record record, cudaGraphExec_t *exec)
+{
+    *exec = nullptr;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
+        cudaGetLastError();
+        return -1;
+    }
+    cudaGraph_t g = nullptr;
+    bool ok = *own || cudaStreamCreateWithFlags(own, cudaStreamNonBlocking) == cudaSuccess;
+    if (ok && cudaStreamBeginCapture(*own, cudaStreamCaptureModeRelaxed) == cudaSuccess) {
+        ok = record(*own) == 0;
+        ok = cudaStreamEndCapture(*own, &g) == cudaSuccess && ok && g &&
+             cudaGraphInstantiate(exec, g, 0) == cudaSuccess;
+    } else {
+        ok = false;
+    }
+    if (g) cudaGraphDestroy(g);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (ok) return 0;
+    cudaGetLastError();
+    *exec = nullptr;
+    return -1;
+}
+
+// True if work enqueued on `s` would go into a capture of the caller's (or if that
+// cannot be told: the launches themselves then report what is wrong).
+inline bool being_captured(cudaStream_t s)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) return false;
+    cudaGetLastError();
+    return true;
+}
+
 // Device state of one time level.
 //  binary64 storage: g = all Q populations [nc][Q][N] (double); the fused
 //    schedule also keeps the densities rhi = [nc][N] (double).
