@@ -48,7 +48,7 @@ struct lbm_batch {
     size_t smem = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
-    cudaGraph_t graph = nullptr;
+    cudaStream_t cap = nullptr;  // where a round is captured: the batch's own stream, or one made for it
     cudaGraphExec_t exec = nullptr;
     int graph_steps = -1;
     double graph_tol = -1.0;
@@ -91,7 +91,7 @@ std::map<std::tuple<int, int, long long>, std::pair<int, size_t>> g_tune_cache;
 void release(lbm_batch *b)
 {
     if (b->exec) cudaGraphExecDestroy(b->exec);
-    if (b->graph) cudaGraphDestroy(b->graph);
+    if (b->cap && !b->own_stream) cudaStreamDestroy(b->cap);
     cudaFree(b->device);
     if (b->pinned) cudaFreeHost(b->pinned);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
@@ -209,21 +209,19 @@ int capture(lbm_batch *b, int steps, double tol)
 {
     if (b->exec && b->graph_steps == steps && b->graph_tol == tol) return LBM_OK;
     if (b->exec) cudaGraphExecDestroy(b->exec);
-    if (b->graph) cudaGraphDestroy(b->graph);
     b->exec = nullptr;
-    b->graph = nullptr;
-    if (cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return LBM_ECUDA;
-    const int st = launch_round(b, steps, tol);
-    cudaGraph_t g = nullptr;
-    if (cudaStreamEndCapture(b->stream, &g) != cudaSuccess || st != LBM_OK) {
-        if (g) cudaGraphDestroy(g);
-        return LBM_ECUDA;
-    }
-    if (cudaGraphInstantiate(&b->exec, g, 0) != cudaSuccess) {
-        cudaGraphDestroy(g);
-        return LBM_ECUDA;
-    }
-    b->graph = g;
+    if (being_captured(b->stream)) return LBM_ECUDA;  // a run waits for its rounds
+    cudaStream_t const user = b->stream;
+    if (b->own_stream) b->cap = b->stream;  // nobody else has it
+    const int st = capture_graph(
+        &b->cap,
+        [&](cudaStream_t s) {
+            b->stream = s;
+            return launch_round(b, steps, tol);
+        },
+        &b->exec);
+    b->stream = user;
+    if (st) return LBM_ECUDA;
     b->graph_steps = steps;
     b->graph_tol = tol;
     return LBM_OK;
@@ -449,9 +447,7 @@ int lbm_batch_set_threads(lbm_batch *b, int threads)
 {
     if (!b || (threads != 128 && threads != 256 && threads != 512)) return LBM_EINVAL;
     if (b->exec) cudaGraphExecDestroy(b->exec);
-    if (b->graph) cudaGraphDestroy(b->graph);
     b->exec = nullptr;
-    b->graph = nullptr;
     b->graph_steps = -1;
     // the shared memory the tuner chose goes with its CTA size; small CTAs need company on their SM
     return configure(b, threads, threads == b->threads ? b->smem_want : 0);

@@ -1,5 +1,6 @@
-"""Problems that share a stream: captured chunks of steps hold the steps of their own
-handle and nothing else, whatever other threads enqueue on the stream meanwhile.
+"""Problems that share a stream: captured chunks of steps, and captured rounds of the
+batched form, hold the work of their own handle and nothing else, whatever other
+threads enqueue on the stream meanwhile.
 
 Every result is bitwise that of the same calls alone: a node's arithmetic depends
 neither on the stream nor on what runs beside it.
@@ -68,6 +69,33 @@ def test_two_handles_of_one_stream_in_two_threads():
                 a, b = together([lambda: run(c, rho, f, st.cuda_stream, start),
                                  lambda: run(c, rho, g, st.cuda_stream, start)])
                 assert np.array_equal(a, alone[f]) and np.array_equal(b, alone[g])
+
+
+@pytest.mark.parametrize("tau", [1.0, 0.8])
+def test_two_batches_of_one_stream_in_two_threads(tau):
+    import torch
+    from paper_2306_10652_gb300 import lbmfug
+    c, _ = mixture()
+    shapes = [(4, 64), (3, 50), (20, 33)]
+    rho = [smooth_rho(490 + k, c, (1,) + s)[:, 0] for k, s in enumerate(shapes)]
+
+    def batch(order, stream, start=None):
+        with lbmfug.Batch(c["a"], c["b"], c["omega"], c["kij"], tau, [(c["T"], rho[k]) for k in order],
+                          stream=stream) as bt:
+            if start is not None:
+                start.wait()
+            for n in (3, 5, 4):  # each another round: captured anew
+                bt.run(max_steps=n, check_every=n, tol=0.0)
+            return {k: bt.state(i)["rho"] for i, k in enumerate(order)}
+
+    alone = batch((0, 1, 2), None)
+    st = torch.cuda.Stream()
+    for _ in range(4):
+        start = threading.Barrier(2)
+        for got in together([lambda: batch((0, 1), st.cuda_stream, start),
+                             lambda: batch((2, 1, 0), st.cuda_stream, start)]):
+            for k, r in got.items():
+                assert np.array_equal(r, alone[k]), k
 
 
 def test_other_work_on_the_stream_runs_once_and_where_it_was_enqueued():
