@@ -335,12 +335,6 @@ void build_par_mu(const lbm_problem *p, df::ParMu &q, df::MuTab &t)
     }
 }
 
-// Host copy of the binary64 logarithm's tables, uploaded once per problem.
-struct Log64Host {
-    Log64 t;
-    Log64Host() { make_log64(&t); }
-};
-
 void build_par64(lbm_problem *p, const Log64 *tab)
 {
     const Params &P = p->P;
@@ -352,7 +346,13 @@ void build_par64(lbm_problem *p, const Log64 *tab)
     q.nc = P.nc;
     q.N = P.N;
     q.RT = P.RT;
-    q.iRT = 1.0 / P.RT;
+    D2 iRT, c2;
+    rt_constants(P.RT, &iRT, &c2);
+    q.iRT = iRT.hi;
+    q.iRTl = iRT.lo;
+    q.c2 = c2.hi;
+    q.c2l = c2.lo;
+    const D2 lnRT = dd_log(P.RT);
     q.omega = P.omega;
     q.tab = tab;
     for (int i = 0; i < P.nc; ++i) {
@@ -363,7 +363,9 @@ void build_par64(lbm_problem *p, const Log64 *tab)
         q.bM[i] = P.b[i] * P.invM[i];
         q.pk[i] = P.sqk[i] * P.invM[i];
         q.kM[i] = q.pk[i] / P.RT;
-        q.c0[i] = P.lnRT + std::log(P.invM[i]);
+        const D2 c0 = dd_add(lnRT, dd_log(P.invM[i]));
+        q.c0[i] = c0.hi;
+        q.c0l[i] = c0.lo;
         for (int j = 0; j < P.nc; ++j) q.A[i * kMaxNc + j] = P.A[i * kMaxNc + j] * P.invM[i] * P.invM[j];
     }
 }
@@ -449,10 +451,9 @@ int ensure_allocated(lbm_problem *p)
     p->w.psi = (double *)dev_alloc(p, (size_t)p->N * sizeof(double));
     p->w.lap = (double *)dev_alloc(p, (size_t)p->N * sizeof(double));
     p->w.jm = (double *)dev_alloc(p, (size_t)p->D * p->N * sizeof(double));
-    static const Log64Host log64_host;
     Log64 *lt = (Log64 *)dev_alloc(p, sizeof(Log64));
     if (!lt) return LBM_ENOMEM;
-    if (cudaMemcpyAsync(lt, &log64_host.t, sizeof(Log64), cudaMemcpyHostToDevice, p->stream) != cudaSuccess)
+    if (cudaMemcpyAsync(lt, &log64_host(), sizeof(Log64), cudaMemcpyHostToDevice, p->stream) != cudaSuccess)
         return LBM_ECUDA;
     build_par64(p, lt);
     if (p->opt.precision == LBM_FP32DEV) {

@@ -67,11 +67,6 @@ const bt::Ops *lookup(int prec, int nc)
     return nullptr;
 }
 
-struct Log64Host {
-    Log64 t;
-    Log64Host() { make_log64(&t); }
-};
-
 double alpha_of(double a, double b, double omega, double T, double R)
 {
     const double Tc = (0.077796074 / 0.457235529) * a / (R * b);  // Sec. 2.3
@@ -312,7 +307,12 @@ int lbm_batch_create(lbm_batch **out, int Nc, const double *a, const double *b, 
         if (!tau1) off += (size_t)Nc * 8 * J.N;
         off = (off + 31) & ~(size_t)31;
         J.RT = o.R * jobs[k].T;
-        J.lnRT = std::log(J.RT);
+        D2 iRT, c2;
+        rt_constants(J.RT, &iRT, &c2);
+        J.iRT = iRT.hi;
+        J.iRTl = iRT.lo;
+        J.c2 = c2.hi;
+        J.c2l = c2.lo;
         double aa[bt::kMaxNcBatch];
         for (int i = 0; i < Nc; ++i) aa[i] = a[i] * alpha_of(a[i], b[i], omega[i], jobs[k].T, o.R);
         for (int i = 0; i < Nc; ++i)
@@ -362,8 +362,7 @@ int lbm_batch_create(lbm_batch **out, int Nc, const double *a, const double *b, 
         *bt_->h_nconv = 0;
     }
     if (!st) {
-        static const Log64Host log64_host;
-        cudaMemcpyAsync(bt_->d_log64, &log64_host.t, sizeof(Log64), cudaMemcpyHostToDevice, bt_->stream);
+        cudaMemcpyAsync(bt_->d_log64, &log64_host(), sizeof(Log64), cudaMemcpyHostToDevice, bt_->stream);
         bt_->S.log64 = bt_->d_log64;
         cudaMemcpyAsync(bt_->d_jobs, bt_->jobs.data(), njobs * sizeof(bt::Job), cudaMemcpyHostToDevice, bt_->stream);
         cudaMemcpyAsync(bt_->d_order, bt_->order.data(), njobs * sizeof(int), cudaMemcpyHostToDevice, bt_->stream);

@@ -111,6 +111,16 @@ int launch_resident(int prec, int nc, const Params &P, const Par64 *p64, const d
     q.N = (int)P.N;
     q.omega = P.omega;
     q.RT = P.RT;
+    D2 iRT, c2;
+    rt_constants(P.RT, &iRT, &c2);
+    auto narrow = [](D2 v) {
+        const float h = (float)v.hi;
+        return make_float2(h, (float)((v.hi - (double)h) + v.lo));
+    };
+    q.iRT = make_double2(iRT.hi, iRT.lo);
+    q.c2 = make_double2(c2.hi, c2.lo);
+    q.fiRT = narrow(iRT);
+    q.fc2 = narrow(c2);
     q.p64 = p64;
     q.pm = pm;
     q.mtab = mtab;

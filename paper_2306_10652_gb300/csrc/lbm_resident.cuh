@@ -41,6 +41,8 @@ struct Par {
     int nx, ny, nc, steps;
     int N;
     double omega, RT;
+    double2 iRT, c2;      // 1 / RT and -1 / (sqrt2 RT) as unevaluated sums,
+    float2 fiRT, fc2;     // in binary32
     const Par64 *p64;     // device copies: binary64 constants,
     const df::ParMu *pm;  // double-binary32 constants
     const df::MuTab *mtab;
@@ -86,7 +88,7 @@ __device__ __forceinline__ double lane_rcp(double x) { return rcp64(x); }
 // mu_i / (M_i RT) up to a constant, and psi: binary32 and binary64 (PrNode of
 // lbm_core.cuh with the components in lanes).
 template <int G, typename E> struct Thermo {
-    E bM, invM, kM, pk, iRT;
+    E bM, invM, kM, pk;
     const E *A;  // shared, [j][G]
     const Log64 *tab;
     __device__ __forceinline__ void init(const Par &P, int i, E *sh, float4 *, float2 *)
@@ -97,7 +99,6 @@ template <int G, typename E> struct Thermo {
         invM = on ? (E)q.invM[i] : (E)0;
         kM = on ? (E)q.kM[i] : (E)0;
         pk = on ? (E)q.pk[i] : (E)0;
-        iRT = (E)q.iRT;
         tab = P.ltab;
         for (int k = threadIdx.x; k < G * G; k += blockDim.x) {
             const int j = k / G, c = k % G;
@@ -106,7 +107,7 @@ template <int G, typename E> struct Thermo {
         A = sh + i;
     }
     __device__ __forceinline__ E psi(E r, float, float) const { return bfly<G>(pk * r); }
-    template <typename At> __device__ __forceinline__ E mu(int nc, bool on, E r, float, float, At psi_at) const
+    template <typename At> __device__ __forceinline__ E mu(const Par &P, bool on, E r, float, float, At psi_at) const
     {
         const E kS2 = (E)1.4142135623730951;
         const E c0 = psi_at(0);
@@ -115,14 +116,20 @@ template <int G, typename E> struct Thermo {
         const E lap = (E)6 * fma((E)(1.0 / 9.0), faces, (E)(1.0 / 36.0) * diags);
         const E B = bfly<G>(bM * r), rho = bfly<G>(invM * r);
         E T = 0;
-        for (int j = 0; j < nc; ++j) T = fma(A[j * G], __shfl_sync(0xffffffffu, r, j, G), T);
+        for (int j = 0; j < P.nc; ++j) T = fma(A[j * G], __shfl_sync(0xffffffffu, r, j, G), T);
         const E Q = bfly<G>(r * T);
-        const E omB = (E)1 - B, den = fma(B, (E)2 - B, (E)1), n1 = fma((E)1 + kS2, B, (E)1);
+        const E omB = (E)1 - B, den = fma(B, (E)2 - B, (E)1);
         const E u = lane_rcp(B), vb = lane_rcp(omB), vd = lane_rcp(den);
-        const E Lu = lane_log(n1 * n1 * vd, tab) * u;
+        const E Lu = lane_log(fma((E)1 + kS2, B, (E)1) * lane_rcp(fma((E)1 - kS2, B, (E)1)), tab) * u;
         const E C0 = -lane_log(omB, tab);
-        const E C1 = fma(Q * (u * iRT), fma((E)0.5 / kS2, Lu, -vd), rho * vb);
-        const E C2 = ((E)-1 / kS2) * iRT * Lu;
+        const E qu = Q * u;
+        E iRT, iRTl, c2, c2l;
+        if constexpr (sizeof(E) == 8)
+            iRT = P.iRT.x, iRTl = P.iRT.y, c2 = P.c2.x, c2l = P.c2.y;
+        else
+            iRT = P.fiRT.x, iRTl = P.fiRT.y, c2 = P.fc2.x, c2l = P.fc2.y;
+        const E C1 = fma(fma(qu, iRT, qu * iRTl), fma((E)0.5 / kS2, Lu, -vd), rho * vb);
+        const E C2 = fma(Lu, c2, Lu * c2l);
         const E lr = lane_log(on ? r : (E)1, tab);
         return fma(invM, lr + C0, fma(bM, C1, fma(T, C2, -kM * lap)));
     }
@@ -171,7 +178,7 @@ template <int G> struct Thermo<G, df::F2> {
         return make_float2(v.hi, v.lo);
     }
     template <typename At>
-    __device__ __forceinline__ float2 mu(int nc, bool on, float, float h, float l, At psi_at) const
+    __device__ __forceinline__ float2 mu(const Par &P, bool on, float, float h, float l, At psi_at) const
     {
         using namespace df;
         constexpr double kS2 = 1.41421356237309504880168872421;
@@ -184,7 +191,7 @@ template <int G> struct Thermo<G, df::F2> {
         const float C12 = __fmul_rn(C, 4097.0f);
         C = __fsub_rn(C12, __fsub_rn(C12, C));
         float s = C, c = 0.0f;
-        for (int j = 0; j < nc; ++j) {
+        for (int j = 0; j < P.nc; ++j) {
             const float2 a = A[j * G];
             const float xh = __shfl_sync(0xffffffffu, h, j, G), xl = __shfl_sync(0xffffffffu, l, j, G);
             const float t = fmaf(a.x, xh, s);
@@ -294,7 +301,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const Par P, StateBufs st,
 #pragma unroll
         for (int a = 0; a < 9; ++a) asm volatile("" : "+r"(nb[a]));
         // P2
-        const R m = th.mu(P.nc, on, r, (float)r, lo, [&](int a) { return __ldcg(psi + nb[a]); });
+        const R m = th.mu(P, on, r, (float)r, lo, [&](int a) { return __ldcg(psi + nb[a]); });
         if (on) __stcg(mu + n * G, m);
         cluster_barrier();
         // P3: the quadratic form in e of lbm_threepass.cuh / lbm_multipass.cuh
