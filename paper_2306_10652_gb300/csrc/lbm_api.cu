@@ -55,7 +55,7 @@ struct lbm_problem {
     double *snap = nullptr;
     bool have_snap = false;
     void *fscratch = nullptr;  // psi / mu scratch of lbm_forces
-    float2 *mu = nullptr;      // [nc][N] grad mu_i of the LBM_FP32DEV step (the mu pass writes it)
+    float2 *mu = nullptr;      // [nc][N] mu_i or grad mu_i of the LBM_FP32DEV step (the mu pass writes it)
     // lbm_step_graph: n steps captured once per starting buffer (cur = 0, 1)
     long long graph_n = 0;
     cudaGraphExec_t graph_exec[2] = {nullptr, nullptr};
@@ -418,20 +418,13 @@ int ensure_allocated(lbm_problem *p)
     if (p->resident) p->fused = p->multipass = false;
     const bool f32 = p->opt.precision != LBM_FP64;
     const size_t nf = (size_t)p->nc * p->N;  // one field per component
-    const bool paired = f32 && (p->multipass || p->fused);
-    const size_t np = paired ? nf + (p->nc & 1) * (size_t)p->N : nf;  // pairs of components
     for (int k = 0; k < 2; ++k) {
         if (f32) {
-            p->st[k].paired = paired;
-            p->st[k].g = dev_alloc(p, np * (p->Q - 1) * sizeof(float));
-            p->st[k].rhi = dev_alloc(p, np * sizeof(float));
-            p->st[k].rlo = (float *)dev_alloc(p, np * sizeof(float));
+            p->st[k].paired = p->multipass || p->fused ? p->nc & ~1 : 0;
+            p->st[k].g = dev_alloc(p, nf * (p->Q - 1) * sizeof(float));
+            p->st[k].rhi = dev_alloc(p, nf * sizeof(float));
+            p->st[k].rlo = (float *)dev_alloc(p, nf * sizeof(float));
             if (!p->st[k].g || !p->st[k].rhi || !p->st[k].rlo) return LBM_ENOMEM;
-            // the partner of an odd last component is empty (k_init and k_from_f64 write st[0]'s)
-            if (np > nf && (cudaMemsetAsync(p->st[k].g, 0, np * (p->Q - 1) * sizeof(float), p->stream) != cudaSuccess ||
-                            cudaMemsetAsync(p->st[k].rhi, 0, np * sizeof(float), p->stream) != cudaSuccess ||
-                            cudaMemsetAsync(p->st[k].rlo, 0, np * sizeof(float), p->stream) != cudaSuccess))
-                return LBM_ECUDA;
             if (p->fused) {
                 p->st[k].j = (float2 *)dev_alloc(p, (size_t)p->N * sizeof(float2));
                 if (!p->st[k].j) return LBM_ENOMEM;
@@ -448,6 +441,7 @@ int ensure_allocated(lbm_problem *p)
     const size_t fb = nf * sizeof(double);
     p->w.rho = (double *)dev_alloc(p, fb);
     p->w.lnf = (double *)dev_alloc(p, fb);
+    p->mu = (float2 *)p->w.lnf;  // LBM_FP32DEV: both live within one step or one call only
     p->w.psi = (double *)dev_alloc(p, (size_t)p->N * sizeof(double));
     p->w.lap = (double *)dev_alloc(p, (size_t)p->N * sizeof(double));
     p->w.jm = (double *)dev_alloc(p, (size_t)p->D * p->N * sizeof(double));
@@ -507,16 +501,12 @@ int ensure_allocated(lbm_problem *p)
         p->mass_parts = (int)parts;
         p->mass_partials = (double *)dev_alloc(p, parts * p->nc * sizeof(double));
         if (!p->mass_partials || p->geo.nstrips < 1) return LBM_ENOMEM;
-        if (p->opt.precision == LBM_FP32DEV) {
-            p->mu = (float2 *)dev_alloc(p, (nf + (p->nc & 1) * p->N) * sizeof(float2));  // grad mu_i (mu pass), pairs
-            if (!p->mu || p->geo.mnstrips < 1) return LBM_ENOMEM;
-        }
+        if (p->opt.precision == LBM_FP32DEV && p->geo.mnstrips < 1) return LBM_ENOMEM;
     }
     if (p->multipass) {
-        p->mu = (float2 *)dev_alloc(p, np * sizeof(float2));
         p->psi2 = (float2 *)dev_alloc(p, (size_t)p->N * sizeof(float2));
         p->jm = (float *)dev_alloc(p, (size_t)p->D * p->N * sizeof(float));
-        if (!p->mu || !p->psi2 || !p->jm) return LBM_ENOMEM;
+        if (!p->psi2 || !p->jm) return LBM_ENOMEM;
     }
     if (cudaMemsetAsync(p->flag, 0, 16, p->stream) != cudaSuccess) return LBM_ECUDA;
     p->allocated = true;

@@ -38,21 +38,23 @@ size_t max_optin_smem()
 }
 
 // j = sum_i sum_a e_a g_{a,i} of a binary32 state (components in pairs)
-__global__ void __launch_bounds__(256) k_momentum(int np, long long N, const float2 *__restrict__ g,
+__global__ void __launch_bounds__(256) k_momentum(int nc, long long N, const void *__restrict__ g,
                                                   float2 *__restrict__ j)
 {
     const long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (r >= N) return;
     float jx = 0.0f, jy = 0.0f;
-    for (int p = 0; p < np; ++p) {
+    auto add = [&](bool one, int p) {
         float2 v[8];
 #pragma unroll
-        for (int a = 0; a < 8; ++a) v[a] = __ldg(g + (p * 8 + a) * N + r);
+        for (int a = 0; a < 8; ++a) v[a] = load_pair(g, one, p, a, 8, N, r);
         jx += (v[0].x - v[1].x) + (v[4].x - v[5].x) + (v[6].x - v[7].x);
         jy += (v[2].x - v[3].x) + (v[4].x - v[5].x) + (v[7].x - v[6].x);
         jx += (v[0].y - v[1].y) + (v[4].y - v[5].y) + (v[6].y - v[7].y);
         jy += (v[2].y - v[3].y) + (v[4].y - v[5].y) + (v[7].y - v[6].y);
-    }
+    };
+    for (int p = 0; p < nc / 2; ++p) add(false, p);
+    if (nc & 1) add(true, nc / 2);
     j[r] = make_float2(jx, jy);
 }
 
@@ -62,25 +64,29 @@ __global__ void __launch_bounds__(256) k_momentum(int np, long long N, const flo
 // pass of its own leaves the shared memory of the step kernel to a third CTA per SM.
 // 2048^2, Nc = 10 (336 MB): 79 us in chunks of 8192 nodes, 85 us in chunks of 2048;
 // below 2^20 nodes the shorter chunks keep the SMs filled.
-__global__ void __launch_bounds__(256) k_mass32(int nc, long long N, const float2 *__restrict__ rhi,
-                                                const float2 *__restrict__ rlo, double *__restrict__ partials)
+__global__ void __launch_bounds__(256) k_mass32(int nc, long long N, const void *__restrict__ rhi,
+                                                const void *__restrict__ rlo, double *__restrict__ partials)
 {
     __shared__ double sh[2][8];
     const int p = blockIdx.y;
     const long long chunk = (N + gridDim.x - 1) / gridDim.x;
     const long long lo = blockIdx.x * chunk;
     const long long hi = lo + chunk < N ? lo + chunk : N;
-    rhi += p * N;
-    rlo += p * N;
     float2 s = make_float2(0.0f, 0.0f), c = s;
+    auto sum = [&](bool one) {
 #pragma unroll 8
-    for (long long r = lo + threadIdx.x; r < hi; r += 256) {
-        const float2 h = __ldg(rhi + r), l = __ldg(rlo + r);
-        acc_add(s.x, c.x, h.x);
-        acc_add(s.y, c.y, h.y);
-        c.x += l.x;
-        c.y += l.y;
-    }
+        for (long long r = lo + threadIdx.x; r < hi; r += 256) {
+            const float2 h = load_pair(rhi, one, p, N, r), l = load_pair(rlo, one, p, N, r);
+            acc_add(s.x, c.x, h.x);
+            c.x += l.x;
+            if (!one) {
+                acc_add(s.y, c.y, h.y);
+                c.y += l.y;
+            }
+        }
+    };
+    if (2 * p + 1 < nc) sum(false);
+    else sum(true);
     double v[2] = {(double)s.x + (double)c.x, (double)s.y + (double)c.y};
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
@@ -190,7 +196,7 @@ int launch_fused_density(int prec, int nc, const Params &P, StateBufs st, cudaSt
 
 int launch_fused_momentum(int nc, long long N, StateBufs st, cudaStream_t s)
 {
-    k_momentum<<<(unsigned)((N + 255) / 256), 256, 0, s>>>((nc + 1) / 2, N, (const float2 *)st.g, st.j);
+    k_momentum<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(nc, N, st.g, st.j);
     return (int)cudaGetLastError();
 }
 
@@ -210,8 +216,7 @@ int launch_fused_mass(int prec, int nc, const Params &P, const FusedGeom &geo, S
     if (prec != 0) {
         const long long b = P.N < (1 << 20) ? (P.N + 2047) / 2048 : (P.N + 8191) / 8192;
         n = (int)(b < parts ? b : parts);
-        k_mass32<<<dim3(n, (nc + 1) / 2), 256, 0, s>>>(nc, P.N, (const float2 *)st.rhi, (const float2 *)st.rlo,
-                                                          partials);
+        k_mass32<<<dim3(n, (nc + 1) / 2), 256, 0, s>>>(nc, P.N, st.rhi, st.rlo, partials);
         *launches = 2;
     }
     k_mass_final<<<nc, 256, 0, s>>>(nc, n, partials, out, nonfinite);

@@ -408,6 +408,19 @@ __device__ __forceinline__ void store_if(bool on, float2 *a, float2 x)
                  "f"(x.x), "f"(x.y), "r"((int)on)
                  : "memory");
 }
+__device__ __forceinline__ void store_if(bool on, float *a, float x)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p st.global.f32 [%0], %1;\n\t}" ::"l"(a), "f"(x),
+                 "r"((int)on)
+                 : "memory");
+}
+// store_pair where `on`
+__device__ __forceinline__ void store_pair_if(bool on, void *base, bool one, int p, int a, int ns, long long N, unsigned o,
+                                              float2 v)
+{
+    if (one) store_if(on, (float *)base + (2LL * p * ns + a) * N + o, v.x);
+    else store_if(on, (float2 *)base + ((long long)p * ns + a) * N + o, v);
+}
 template <typename E> constexpr int wmax32() { return kT - 2 * (std::is_same<E, DF64>::value ? 2 : 3); }
 
 // asynchronous copies to shared memory (no register holds the data in flight)
@@ -418,6 +431,12 @@ template <int BYTES> __device__ __forceinline__ void copy_async(void *dst, const
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
     else
         asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES) : "memory");
+}
+// node o of pair p into *dst (an odd last component: into its first word)
+__device__ __forceinline__ void copy_pair(float2 *dst, const void *base, bool one, int p, long long N, unsigned o)
+{
+    if (one) copy_async<4>(dst, (const float *)base + 2LL * p * N + o);
+    else copy_async<8>(dst, (const float2 *)base + (long long)p * N + o);
 }
 __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -431,8 +450,8 @@ __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_
 //   grad mu(k-2) on the interior columns from mu rows k-3..k-1, every
 //     difference mu(r + e) - mu(r - e) taken on the (hi, lo) pairs and
 //     rounded once (so it carries the df64 accuracy of mu), written in binary32
-//     to G[p][node], (d/dx, d/dx, d/dy, d/dy) of components 2p and 2p + 1 (an
-//     odd last component is paired with zeros).
+//     to G[p][node], (d/dx, d/dx, d/dy, d/dy) of components 2p and 2p + 1, or
+//     (d/dx, d/dy) of an odd last one.
 // The step kernel forms F_i = -rho~_i G_i.  psi and mu rows live in rings of
 // three: a slot is rewritten only after the barrier that follows its last
 // reader.
@@ -458,6 +477,7 @@ __global__ void __launch_bounds__(kT, NC <= 10 ? 4 : 3)
     k_mu32(const df::ParMu P, const int W, const int H, StateBufs in, float4 *__restrict__ G)
 {
     constexpr int NP = SmemMu<NC>::NP, CW = NP * kT;
+    auto one = [](int p) { return 2 * p + 1 == NC; };  // an odd last component
     extern __shared__ __align__(16) unsigned char smem[];
     float4 *TV = (float4 *)smem;      // [128] logarithm tables
     float2 *TK = (float2 *)(TV + 128);  // [512]
@@ -476,15 +496,13 @@ __global__ void __launch_bounds__(kT, NC <= 10 ? 4 : 3)
     const bool hasM = c >= -1 && c <= w;
     const bool interior = c >= 0 && c < w;
     const unsigned xg = (unsigned)wrapc(x0 + c, nx);
-    const float2 *__restrict__ rhin = (const float2 *)in.rhi;
-    const float2 *__restrict__ rlin = (const float2 *)in.rlo;
     df::load_mu_tab(P.tab, TV, TK);
     auto copy_row = [&](int y) {  // asynchronous, the thread's own column
         const unsigned o = (unsigned)wrapc(y, ny) * (unsigned)nx + xg;
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-            copy_async<8>(NX + p * kT + t, rhin + p * N + o);
-            copy_async<8>(NX + (NP + p) * kT + t, rlin + p * N + o);
+            copy_pair(NX + p * kT + t, in.rhi, one(p), p, N, o);
+            copy_pair(NX + (NP + p) * kT + t, in.rlo, one(p), p, N, o);
         }
     };
     if (hasP) copy_row(y0 - 2);
@@ -502,7 +520,7 @@ __global__ void __launch_bounds__(kT, NC <= 10 ? 4 : 3)
             for (int p = 0; p < NP; ++p) {
                 const float2 a = NX[p * kT + t], b = NX[(NP + p) * kT + t];
                 hh[2 * p] = a.x, ll[2 * p] = b.x;
-                if (2 * p + 1 < NC) hh[2 * p + 1] = a.y, ll[2 * p + 1] = b.y;
+                if (!one(p)) hh[2 * p + 1] = a.y, ll[2 * p + 1] = b.y;
             }
             df::F2 ps;
             df::psi_and_B<NC>(P, hh, ll, ps, Bk);
@@ -545,7 +563,8 @@ __global__ void __launch_bounds__(kT, NC <= 10 ? 4 : 3)
                 const float2 f = df::vbc(1.0f / 9.0f), d = df::vbc(1.0f / 36.0f), three = df::vbc(3.0f);
                 const float2 gx = df::vmul(three, df::vfma(f, dE, df::vmul(d, df::vadd(dNE, dSE))));
                 const float2 gy = df::vmul(three, df::vfma(f, dN, df::vmul(d, df::vsub(dNE, dSE))));
-                G[p * N + ob] = make_float4(gx.x, gx.y, gy.x, gy.y);
+                if (one(p)) ((float2 *)(G + p * N))[ob] = make_float2(gx.x, gy.x);
+                else G[p * N + ob] = make_float4(gx.x, gx.y, gy.x, gy.y);
             }
         }
     }
@@ -553,8 +572,8 @@ __global__ void __launch_bounds__(kT, NC <= 10 ? 4 : 3)
 
 // Binary32 state: the 8 moving populations (a = 1..8), the density rho_i = hi + lo
 // and the momentum j = sum_i sum_a e_a g_{a,i}; components in pairs, g[p][a-1][node][2]
-// and rhi, rlo[p][node][2], so that a load or store serves two.  Collision
-// arithmetic in binary32; thermodynamics and forces in E.  The new density of a
+// and rhi, rlo[p][node][2], so that a load or store serves two (an odd last one alone,
+// StateBufs).  Collision arithmetic in binary32; thermodynamics and forces in E.  The new density of a
 // node is its old density minus the populations that left it plus those that
 // arrived: every stored binary32 population is added once where it arrives and
 // subtracted once where it left, each by an error-free Fast2Sum into the (hi, lo)
@@ -588,9 +607,9 @@ __global__ void __launch_bounds__(kT, NC <= 10 ? 4 : 3)
 // per SM, 0.134 ms with three, 0.141 ms with three and the components apart, 0.260 ms
 // at first; Nc = 10 needs more than the 128 registers that four leave it.
 template <int NC, typename E, bool TAU1>
-__global__ void __launch_bounds__(kT, NC <= 6 ? 4 : NC <= 10 ? 3 : 2)
+__global__ void __launch_bounds__(kT, NC == 1 ? 6 : NC <= 6 ? 4 : NC <= 10 ? 3 : 2)
     k_fused32(const Par32 P, const int W, const int H, StateBufs in, StateBufs out,
-              const float4 *__restrict__ mug /* DF64: grad mu of a pair of components (x, x, y, y) */)
+              const float4 *__restrict__ mug /* DF64: grad mu of a pair of components (x, x, y, y); an odd last one (x, y) */)
 {
     using L = Lattice<0>;
     using SM = Smem32<NC, E>;
@@ -601,6 +620,7 @@ __global__ void __launch_bounds__(kT, NC <= 6 ? 4 : NC <= 10 ? 3 : 2)
     constexpr bool kDF = SM::kDF;
     constexpr int NP = SM::NP, kHalo = SM::kHalo, kRing = SM::kRing, kLag = kDF ? 1 : 2;
     constexpr int CW = NP * kT;  // a ring slot
+    auto one = [](int p) { return 2 * p + 1 == NC; };  // an odd last component
     extern __shared__ __align__(16) unsigned char smem[];
     float2 *RS = (float2 *)smem;                              // [kRing][NP][kT] rho hi rows
     float4 *GS = (float4 *)(RS + kRing * CW);                 // [NP][kT] grad mu of row q
@@ -609,12 +629,12 @@ __global__ void __launch_bounds__(kT, NC <= 6 ? 4 : NC <= 10 ? 3 : 2)
     float2 *JS = XC + 6 * CW;                                 // [kT] momentum of row q
     float *XJ = (float *)(JS + kT);                           // [6][kT]
     float *PS = XJ + 6 * kT;                                  // [3][kT] psi rows (binary32)
-    const float2 *__restrict__ gin = (const float2 *)in.g;
-    float2 *__restrict__ gout = (float2 *)out.g;
-    const float2 *__restrict__ rhin = (const float2 *)in.rhi;
-    const float2 *__restrict__ rlin = (const float2 *)in.rlo;
-    float2 *__restrict__ rhout = (float2 *)out.rhi;
-    float2 *__restrict__ rlout = (float2 *)out.rlo;
+    const void *__restrict__ gin = in.g;
+    void *__restrict__ gout = out.g;
+    const void *__restrict__ rhin = in.rhi;
+    const void *__restrict__ rlin = in.rlo;
+    void *__restrict__ rhout = out.rhi;
+    void *__restrict__ rlout = out.rlo;
     const float2 *__restrict__ jin = in.j;
     float2 *__restrict__ jout = out.j;
 
@@ -649,21 +669,30 @@ __global__ void __launch_bounds__(kT, NC <= 6 ? 4 : NC <= 10 ? 3 : 2)
     // asynchronous copies of the thread's own column
     auto copy_density = [&](int y, int slot) {
         if (!loads) return;
-        const float2 *src = rhin + row(y) + xg;
+        const unsigned o = row(y) + xg;
         float2 *dst = RS + slot * CW + t;
 #pragma unroll
-        for (int p = 0; p < NP; ++p) copy_async<8>(dst + p * kT, src + p * N);
+        for (int p = 0; p < NP; ++p) copy_pair(dst + p * kT, rhin, one(p), p, N, o);
     };
     auto copy_collision = [&](int y) {
         if (!active) return;
         const unsigned o = row(y) + xg;
         copy_async<8>(JS + t, jin + o);
-        if constexpr (kDF)
+        if constexpr (kDF) {
 #pragma unroll
-            for (int p = 0; p < NP; ++p) copy_async<16>(GS + p * kT + t, mug + p * N + o);
+            for (int p = 0; p < NP; ++p) {
+                if (one(p)) copy_async<8>(GS + p * kT + t, (const float2 *)(mug + p * N) + o);
+                else copy_async<16>(GS + p * kT + t, mug + p * N + o);
+            }
+        }
     };
 
-    // (an odd last component shares its operations with an empty one, zero in the state)
+    // an odd last component shares its operations with a zero: the copies leave its words
+    // in the density rows alone
+    if constexpr (NC & 1) {
+#pragma unroll
+        for (int k = 0; k < kRing; ++k) RS[k * CW + (NP - 1) * kT + t].y = 0.0f;
+    }
     if (!loads)  // columns beyond the strip feed psi rows only
 #pragma unroll
         for (int p = 0; p < kRing * NP; ++p) RS[p * kT + t] = vbc(0.0f);
@@ -748,9 +777,15 @@ __global__ void __launch_bounds__(kT, NC <= 6 ? 4 : NC <= 10 ? 3 : 2)
                 const float2 cr = vmul(P.cf[p], ri);
                 float2 gx, gy;
                 if constexpr (kDF) {
-                    const float4 g = GS[p * kT + t];
-                    gx = make_float2(g.x, g.y);
-                    gy = make_float2(g.z, g.w);
+                    if (one(p)) {
+                        const float2 g = *(const float2 *)(GS + p * kT + t);
+                        gx = make_float2(g.x, 0.0f);
+                        gy = make_float2(g.y, 0.0f);
+                    } else {
+                        const float4 g = GS[p * kT + t];
+                        gx = make_float2(g.x, g.y);
+                        gy = make_float2(g.z, g.w);
+                    }
                 } else {
                     const int q1 = (kk + 1) % 3;  // mu row q = k-2
                     grad12(MU + ((q1 + 2) % 3) * CW + p * kT + t, MU + q1 * CW + p * kT + t,
@@ -782,7 +817,7 @@ __global__ void __launch_bounds__(kT, NC <= 6 ? 4 : NC <= 10 ? 3 : 2)
                 float2 v[9];
                 if constexpr (!TAU1) {
 #pragma unroll
-                    for (int a = 1; a < 9; ++a) v[a] = __ldg(gin + (8 * p + a - 1) * N + rc);
+                    for (int a = 1; a < 9; ++a) v[a] = load_pair(gin, one(p), p, a - 1, 8, N, rc);
                 }
                 float2 Gx, Gy;
                 grad12(R0 + p * kT, R1 + p * kT, R2 + p * kT, Gx, Gy);
@@ -806,7 +841,7 @@ __global__ void __launch_bounds__(kT, NC <= 6 ? 4 : NC <= 10 ? 3 : 2)
                         g = vfma(vbc(P.om1), v[a], g);
                         S[a] = vadd(S[a], g);
                     }
-                    store_if(st, gout + (8 * p + a - 1) * N + dst[a], g);
+                    store_pair_if(st, gout, one(p), p, a - 1, 8, N, dst[a], g);
                     leave(bH[p], bL[p], g);
                     const int ex = L::e(a, 0), ey = L::e(a, 1);
                     if (ex != 0) X[((ey + 1) * 2 + (ex > 0 ? 0 : 1)) * CW] = g;
@@ -891,8 +926,8 @@ __global__ void __launch_bounds__(kT, NC <= 6 ? 4 : NC <= 10 ? 3 : 2)
                 arrive(aH[p], aL[p], X[1 * CW + 1]);
                 const float2 hi = vadd(aH[p], aL[p]);
                 const float2 lo = vfma(vfma(aH[p], m1, hi), m1, aL[p]);
-                store_if(write_row, rhout + p * N + rw, hi);
-                store_if(write_row, rlout + p * N + rw, lo);
+                store_pair_if(write_row, rhout, one(p), p, 0, 1, N, rw, hi);
+                store_pair_if(write_row, rlout, one(p), p, 0, 1, N, rw, lo);
                 aH[p] = bH[p];
                 aL[p] = bL[p];
                 arrive(aH[p], aL[p], X[2 * CW - 1]);
@@ -908,7 +943,7 @@ __global__ void __launch_bounds__(kT, NC <= 6 ? 4 : NC <= 10 ? 3 : 2)
         if (interior && kk + 1 < nrows && kk + 1 >= 2 * kLag) {
             const unsigned o = row(crow + 2) + xg;
 #pragma unroll
-            for (int p = 0; p < NP; ++p) nL[p] = __ldg(rlin + p * N + o);
+            for (int p = 0; p < NP; ++p) nL[p] = load_pair(rlin, one(p), p, N, o);
         }
     }
 }

@@ -115,18 +115,45 @@ struct StateBufs {
     void *rhi = nullptr;
     float *rlo = nullptr;
     float2 *j = nullptr;
-    // binary32, multi-pass and fused schedules: components in pairs, g[p][a][N][2] and
-    // rhi, rlo [p][N][2] (component 2p + k at element k; nc rounded up to even)
+    // binary32, multi-pass and fused schedules: this many components (an even number)
+    // are stored in pairs, g[p][a][N][2] and rhi, rlo [p][N][2] (component 2p + k at
+    // element k).  An odd last component follows alone, g[a][N] and rhi, rlo [N], which
+    // is where it stands without pairs: it shares its packed operations with a zero that
+    // no array holds.  (Paired with a stored zero, a state of Nc = 1 took twice its
+    // bytes, and that zero turned into NaN with a diverged run.)
     int paired = 0;
     // element of component i, slot a of ns at node r
     __host__ __device__ long long at(int i, int a, int ns, long long N, long long r) const
     {
-        return paired ? (((long long)(i >> 1) * ns + a) * N + r) * 2 + (i & 1) : ((long long)i * ns + a) * N + r;
+        return i < paired ? (((long long)(i >> 1) * ns + a) * N + r) * 2 + (i & 1) : ((long long)i * ns + a) * N + r;
     }
     __host__ __device__ long long at(int i, long long N, long long r) const { return at(i, 0, 1, N, r); }
     __host__ __device__ float *rhi_f() const { return (float *)rhi; }
     __host__ __device__ double *rhi_d() const { return (double *)rhi; }
 };
+
+// Node o of plane a (of ns) of pair p of components; `one`: an odd last component,
+// stored alone, beside a zero.  (A constant where these are called.)
+__device__ __forceinline__ float2 load_pair(const void *base, bool one, int p, int a, int ns, long long N, long long o)
+{
+    if (one) return make_float2(__ldg((const float *)base + (2LL * p * ns + a) * N + o), 0.0f);
+    return __ldg((const float2 *)base + ((long long)p * ns + a) * N + o);
+}
+__device__ __forceinline__ float2 load_pair(const void *base, bool one, int p, long long N, long long o)
+{
+    return load_pair(base, one, p, 0, 1, N, o);
+}
+__device__ __forceinline__ void store_pair(void *base, bool one, int p, int a, int ns, long long N, long long o, float2 v)
+{
+    if (one)
+        ((float *)base)[(2LL * p * ns + a) * N + o] = v.x;
+    else
+        ((float2 *)base)[((long long)p * ns + a) * N + o] = v;
+}
+__device__ __forceinline__ void store_pair(void *base, bool one, int p, long long N, long long o, float2 v)
+{
+    store_pair(base, one, p, 0, 1, N, o, v);
+}
 
 // Scratch fields of the three-pass schedule (device).
 struct ThreePassWork {
@@ -181,8 +208,8 @@ FusedGeom fused_geometry_forced(int prec, int nc, const Params &P, int num_sms, 
 int launch_fused_density(int prec, int nc, const Params &P, StateBufs st, cudaStream_t s);
 // binary32 only: momentum of the state from its populations
 int launch_fused_momentum(int nc, long long N, StateBufs st, cudaStream_t s);
-// mu: grad mu_i of LBM_FP32DEV, nc (rounded up to even) x N (else unused); *launches receives the
-// kernels launched.
+// mu: grad mu_i of LBM_FP32DEV, nc x N (else unused); *launches receives the kernels
+// launched.
 int launch_fused_step(int prec, int nc, const Params &P, const df::ParMu &pm, const FusedGeom &geo, StateBufs in,
                       StateBufs out, double *mass_partials, float2 *mu, int *launches, KernelTimer *kt,
                       cudaStream_t s);
@@ -192,8 +219,8 @@ int launch_fused_mass(int prec, int nc, const Params &P, const FusedGeom &geo, S
                       int parts, double *out, int *nonfinite, int *launches, cudaStream_t s);
 
 // Binary32 multi-pass schedule of LBM_FP32DEV on any lattice
-// (lbm_multipass.cu): psi [N] (hi, lo) of the current state, mu (nc rounded up to
-// even) x N (hi, lo) scratch, jm [D][N] momentum of the current state.
+// (lbm_multipass.cu): psi [N] (hi, lo) of the current state, mu nc x N (hi, lo)
+// scratch, jm [D][N] momentum of the current state.
 bool multipass_supported(int lat, int prec, int nc, long long N);
 int launch_multipass_psi(int lat, int nc, const Params &P, const df::ParMu &pm, StateBufs st, float2 *psi, float *jm,
                          cudaStream_t s);

@@ -55,10 +55,8 @@ size_t estimate_bytes(int lattice, long long N, int nc, int precision)
     const int Q = lattice == LBM_D2Q9 ? 9 : 19;
     const int D = lattice == LBM_D2Q9 ? 2 : 3;
     const size_t f = (size_t)nc * N;
-    // the multi-pass and fused schedules keep the state and mu in pairs of components
-    const size_t f2 = precision == LBM_FP32DEV || (precision == LBM_FP32 && lattice == LBM_D2Q9) ? (size_t)(nc + (nc & 1)) * N : f;
-    size_t b = (precision == LBM_FP64) ? 2 * f * Q * 8 + 2 * f * 8 : 2 * f2 * ((Q - 1) * 4 + 8) + 2 * f * 4;
-    if (precision != LBM_FP64) b += f2 * 8 + (size_t)N * 8;  // grad mu (or mu) pairs, psi pairs
+    size_t b = (precision == LBM_FP64) ? 2 * f * Q * 8 + 2 * f * 8 : 2 * f * ((Q - 1) * 4 + 8) + 2 * f * 4;
+    if (precision != LBM_FP64) b += f * 8 + (size_t)N * 8;  // momentum, psi pairs
     b += 2 * f * 8 + (size_t)N * 8 * (2 + D);  // three-pass scratch fields
     b += f * 8;                                 // convergence snapshot
     // reductions and launch tables, plus the device allocator's rounding of

@@ -128,12 +128,11 @@ __global__ void __launch_bounds__(kThreads)
             B[a] = 3.0 * ue + 4.5 * ue * ue - 1.5 * u2;
         }
     }
-    if (sizeof(S) == 4 && st.paired) {  // both components of a pair with one store
+    if (sizeof(S) == 4) {  // both components of a pair with one store
         float2 *g2 = (float2 *)st.g, *rh2 = (float2 *)st.rhi, *rl2 = (float2 *)st.rlo;
 #pragma unroll 2
-        for (int p = 0; p < (nc + 1) / 2; ++p) {
-            const bool two = 2 * p + 1 < nc;
-            const double r0 = __ldg(rho + 2 * p * N + r), r1 = two ? __ldg(rho + (2 * p + 1) * N + r) : 0.0;
+        for (int p = 0; p < st.paired / 2; ++p) {
+            const double r0 = __ldg(rho + 2 * p * N + r), r1 = __ldg(rho + (2 * p + 1) * N + r);
 #pragma unroll
             for (int a = 1; a < L::Q; ++a)
                 g2[(p * NS + a - 1) * N + r] = u ? make_float2((float)(L::w(a) * r0 * B[a]), (float)(L::w(a) * r1 * B[a]))
@@ -142,10 +141,9 @@ __global__ void __launch_bounds__(kThreads)
             rh2[p * N + r] = hi;
             rl2[p * N + r] = make_float2((float)(r0 - (double)hi.x), (float)(r1 - (double)hi.y));
         }
-        return;
     }
 #pragma unroll 2
-    for (int i = 0; i < nc; ++i) {
+    for (int i = st.paired; i < nc; ++i) {
         const double ri = __ldg(rho + i * N + r);
 #pragma unroll
         for (int a = 0; a < L::Q; ++a) {
@@ -180,16 +178,17 @@ __global__ void __launch_bounds__(kThreads)
     const long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (r >= N) return;
     if constexpr (!kFull && sizeof(S) == 4) {
-        if (st.paired) {  // both components of a pair with one load
-            const float2 *__restrict__ h2 = (const float2 *)st.rhi, *__restrict__ l2 = (const float2 *)st.rlo;
+        // both components of a pair with one load
+        const float2 *__restrict__ h2 = (const float2 *)st.rhi, *__restrict__ l2 = (const float2 *)st.rlo;
 #pragma unroll 4
-            for (int p = 0; p < (P.nc + 1) / 2; ++p) {
-                const float2 h = __ldg(h2 + p * N + r), l = __ldg(l2 + p * N + r);
-                rho[2 * p * N + r] = widen(h.x) + widen(l.x);
-                if (2 * p + 1 < P.nc) rho[(2 * p + 1) * N + r] = widen(h.y) + widen(l.y);
-            }
-            return;
+        for (int p = 0; p < st.paired / 2; ++p) {
+            const float2 h = __ldg(h2 + p * N + r), l = __ldg(l2 + p * N + r);
+            rho[2 * p * N + r] = widen(h.x) + widen(l.x);
+            rho[(2 * p + 1) * N + r] = widen(h.y) + widen(l.y);
         }
+#pragma unroll 2
+        for (int i = st.paired; i < P.nc; ++i) rho[i * N + r] = widen(__ldg(rh + i * N + r)) + widen(__ldg(rl + i * N + r));
+        return;
     }
     // momentum: binary64 storage sums the differences of opposite directions over
     // all components, binary32 storage each component in binary32 first
@@ -525,14 +524,6 @@ __global__ void k_from_f64(const Params P, const double *__restrict__ in, StateB
                 st.rhi_f()[st.at(i, N, r)] = hi;
                 st.rlo[st.at(i, N, r)] = (float)(rho - (double)hi);
             }
-        }
-        // the empty partner of an odd last component: what the state held before may
-        // not be finite, and the passes sum over both components of a pair
-        if (sizeof(S) == 4 && (NC & 1) && st.paired) {
-#pragma unroll
-            for (int k = 0; k < NS; ++k) g[st.at(NC, k, NS, N, r)] = (S)0;
-            st.rhi_f()[st.at(NC, N, r)] = 0.0f;
-            st.rlo[st.at(NC, N, r)] = 0.0f;
         }
     }
 }
