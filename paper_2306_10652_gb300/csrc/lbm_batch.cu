@@ -79,9 +79,24 @@ double alpha_of(double a, double b, double omega, double T, double R)
     return s * s;
 }
 
-// autotuner cache: (precision, nc, max nodes) -> (threads, shared memory) per CTA
+// autotuner cache: what the best (threads, shared memory) per CTA depends on: device,
+// precision, Nc, the kernel (tau = 1 or not), the largest box, jobs per SM (how many CTAs
+// should share one, up to four) and how far the boxes fill the largest on average (in
+// quarters; smaller ones keep their exchange buffer on chip in less)
+using TuneKey = std::tuple<int, int, int, bool, long long, int, int>;
 std::mutex g_tune_mutex;
-std::map<std::tuple<int, int, long long>, std::pair<int, size_t>> g_tune_cache;
+std::map<TuneKey, std::pair<int, size_t>> g_tune_cache;
+
+TuneKey tune_key(const lbm_batch *b)
+{
+    int dev = 0, nsm = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    long long nodes = 0;
+    for (const bt::Job &J : b->jobs) nodes += J.N;
+    return TuneKey(dev, b->precision, b->nc, b->S.omega == 1.0, b->maxN, std::min((b->njobs + nsm - 1) / nsm, 4),
+                   (int)(4 * nodes / (b->njobs * b->maxN)));
+}
 
 void release(lbm_batch *b)
 {
@@ -146,7 +161,7 @@ std::vector<size_t> smem_candidates(const lbm_batch *b)
 // Time one short round per candidate on a copy of the state, keep the fastest.
 int autotune(lbm_batch *b)
 {
-    const auto key = std::make_tuple(b->precision, b->nc, b->maxN);
+    const TuneKey key = tune_key(b);
     {
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         auto it = g_tune_cache.find(key);

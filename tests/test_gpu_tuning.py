@@ -1,0 +1,26 @@
+"""What the launch-geometry tuners remember: a choice serves the problems that run the
+same kernel at the same load, and no others.  Trials are launches, which are counted."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from helpers import gpu_problem, seeded_mixture, smooth_rho
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("precision", [2, 1], ids=["fp32", "fp32dev"])
+def test_batch_tuner_knows_kernel_and_load(precision):
+    from paper_2306_10652_gb300 import lbmfug
+    nc, shape = 2, (1, 3, 37 + precision)
+    c = seeded_mixture(510, nc, 0, shape)
+    rho = smooth_rho(510, c, shape)[:, 0]
+
+    def trials(njobs, tau):
+        with lbmfug.Batch(c["a"], c["b"], c["omega"], c["kij"], tau, [(c["T"], rho)] * njobs, precision=precision) as b:
+            return b.info()["launches"]
+
+    for njobs, tau in ((8, 1.0), (700, 1.0), (8, 0.8), (700, 0.8)):  # one job per SM, and four or more
+        assert trials(njobs, tau) > 0, (njobs, tau)
+        assert trials(njobs, tau) == 0, (njobs, tau)
