@@ -117,7 +117,7 @@ typedef struct lbm_options {
                              candidate launch geometries (strips per row, segment
                              waves, mu-pass waves) on the problem itself and keeps
                              the fastest, cached for the process by (precision, Nc,
-                             nx, ny); 0 = the built-in geometry.  The geometry does
+                             nx, ny, tau = 1 or not); 0 = the built-in geometry.  The geometry does
                              not change any result (every node's arithmetic is the
                              same); the first lbm_step then synchronises once. */
     int strip;            /* > 0: interior columns per CTA of the fused kernel (forces

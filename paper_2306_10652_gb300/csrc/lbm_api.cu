@@ -526,9 +526,10 @@ std::vector<TuneCand> tune_candidates(const lbm_problem *p)
 
 struct TuneKey {
     int prec, nc, nx, ny;
+    bool tau1;  // the step kernel of tau = 1 is another one
     bool operator<(const TuneKey &o) const
     {
-        return std::tie(prec, nc, nx, ny) < std::tie(o.prec, o.nc, o.nx, o.ny);
+        return std::tie(prec, nc, nx, ny, tau1) < std::tie(o.prec, o.nc, o.nx, o.ny, o.tau1);
     }
 };
 std::mutex g_tune_mutex;
@@ -538,7 +539,7 @@ std::map<TuneKey, TuneCand> g_tune_cache;
 // st[cur] -> st[cur ^ 1] without swapping, so the state is untouched.
 int tune_geometry(lbm_problem *p)
 {
-    const TuneKey key{p->opt.precision, p->nc, p->nx, p->ny};
+    const TuneKey key{p->opt.precision, p->nc, p->nx, p->ny, p->P.omega == 1.0};
     TuneCand best{0, 1, 1};
     bool cached = false;
     {

@@ -147,7 +147,7 @@ FusedGeom fused_geometry(int prec, int nc, const Params &P, int num_sms, int ext
     g.strip = (P.nx + g.nstrips - 1) / g.nstrips;   // balanced strip width <= wmax
     g.nstrips = (P.nx + g.strip - 1) / g.strip;
     g.smem = o->smem(g.strip);
-    int per_sm = o->occupancy(g.smem);
+    int per_sm = o->occupancy(P.omega == 1.0, g.smem);
     if (per_sm < 1) per_sm = 1;
     const long long slots = (long long)num_sms * per_sm * (seg_mult > 0 ? seg_mult : 1);
     long long segs = slots / g.nstrips;

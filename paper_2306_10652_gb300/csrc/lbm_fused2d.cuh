@@ -973,7 +973,7 @@ struct Ops {
     int (*step)(const Params &, const df::ParMu &, const FusedGeom &, StateBufs, StateBufs, double *, float2 *mu, int *launches,
                 KernelTimer *, cudaStream_t);
     size_t (*smem)(int W);
-    int (*occupancy)(size_t smem);
+    int (*occupancy)(bool tau1, size_t smem);  // CTAs per SM of the step kernel that will run
     int (*occupancy_mu)();  // CTAs per SM of the mu pass (0: the form has none)
 };
 
@@ -982,10 +982,10 @@ struct Ops {
 template <int NC, typename S, typename E> struct Impl {
     static constexpr bool k64 = sizeof(S) == 8;
     static constexpr bool kDF = std::is_same<E, DF64>::value;
-    static auto kernel()
+    static auto kernel(bool tau1)
     {
         if constexpr (k64) return k_fused<NC, double, double>;
-        else return k_fused32<NC, E, false>;
+        else return tau1 ? k_fused32<NC, E, true> : k_fused32<NC, E, false>;
     }
     static constexpr int wmax()
     {
@@ -1006,19 +1006,15 @@ template <int NC, typename S, typename E> struct Impl {
         if constexpr (k64) return Smem<NC, double, double>::total(W);
         else return Smem32<NC, E>::total();
     }
-    static int occupancy(size_t bytes)
+    static int occupancy(bool tau1, size_t bytes)
     {
         // the limit is the widest strip's need, so that problems of other
         // widths launched later keep fitting under it
-        if (cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(kernel(tau1), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem(wmax())) != cudaSuccess)
             return 0;
-        if constexpr (!k64)
-            if (cudaFuncSetAttribute(k_fused32<NC, E, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem(wmax())) != cudaSuccess)
-                return 0;
         int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel(), kT, bytes) != cudaSuccess)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel(tau1), kT, bytes) != cudaSuccess)
             return 0;
         return n;
     }
@@ -1057,7 +1053,7 @@ template <int NC, typename S, typename E> struct Impl {
                 *launches = 2;
             }
             const Par32 q = make_par32(P, kDF);
-            auto step32 = P.omega == 1.0 ? k_fused32<NC, E, true> : k_fused32<NC, E, false>;
+            auto step32 = kernel(P.omega == 1.0);
             kt_begin(kt, kKtStep, s);
             step32<<<grid, kT, g.smem, s>>>(q, g.strip, g.seg_h, in, out, (const float4 *)mu);
             kt_end(kt, s);

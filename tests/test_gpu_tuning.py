@@ -24,3 +24,23 @@ def test_batch_tuner_knows_kernel_and_load(precision):
     for njobs, tau in ((8, 1.0), (700, 1.0), (8, 0.8), (700, 0.8)):  # one job per SM, and four or more
         assert trials(njobs, tau) > 0, (njobs, tau)
         assert trials(njobs, tau) == 0, (njobs, tau)
+
+
+@pytest.mark.parametrize("precision,launches", [(2, 1), (1, 2)], ids=["fp32", "fp32dev"])
+def test_step_tuner_knows_the_kernel(precision, launches):
+    nc, shape = 3, (1, 22, 150 + precision)
+    c = seeded_mixture(515, nc, 0, shape, Tfac=1.2)
+    rho = smooth_rho(515, c, shape)
+
+    def first_step(tau):
+        with gpu_problem(c, 0, shape, tau=tau, precision=precision, schedule=2) as gp:
+            gp.init_fields(rho)
+            n = gp.launch_count()
+            gp.step(1)
+            return gp.launch_count() - n, gp.get_state()
+
+    for tau in (1.0, 0.8):
+        n, tuned = first_step(tau)
+        assert n > launches, tau
+        n, again = first_step(tau)
+        assert n == launches and np.array_equal(tuned, again), tau
