@@ -343,7 +343,8 @@ int lbm_batch_job_state(lbm_batch *b, int job, double *rho, long long *steps, do
 int lbm_batch_info(const lbm_batch *b, int *threads, int *ctas, long long *rounds,
                    long long *launches);
 
-/* Override the CTA size (128, 256 or 512 threads). */
+/* Override the CTA size (128, 256 or 512 threads, or the size that the tuner chose,
+ * which lbm_batch_info reports after creation). */
 int lbm_batch_set_threads(lbm_batch *b, int threads);
 
 int lbm_batch_destroy(lbm_batch *b);

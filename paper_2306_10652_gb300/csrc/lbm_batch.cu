@@ -42,7 +42,7 @@ struct lbm_batch {
     size_t pool_floats = 0;
     long long maxN = 0;
     Log64 *d_log64 = nullptr;
-    size_t smem_want = 0;    // shared memory per CTA the tuner chose
+    std::pair<int, size_t> tuned{0, 0};  // threads and shared memory per CTA that the tuner chose
     const bt::Ops *ops = nullptr;
     int threads = 0, ctas = 0;
     size_t smem = 0;
@@ -134,7 +134,6 @@ int configure(lbm_batch *b, int threads, size_t want)
     if (per_sm < 1) return LBM_ENOTSUP;
     b->threads = threads;
     b->smem = smem;
-    b->smem_want = want;
     b->ctas = std::min((long long)nsm * per_sm, (long long)b->njobs);
     return LBM_OK;
 }
@@ -165,7 +164,10 @@ int autotune(lbm_batch *b)
     {
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         auto it = g_tune_cache.find(key);
-        if (it != g_tune_cache.end()) return configure(b, it->second.first, it->second.second);
+        if (it != g_tune_cache.end()) {
+            b->tuned = it->second;
+            return configure(b, b->tuned.first, b->tuned.second);
+        }
     }
     float *backup = nullptr;
     bt::Status *sbackup = nullptr;
@@ -212,6 +214,7 @@ int autotune(lbm_batch *b)
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         g_tune_cache[key] = best;
     }
+    b->tuned = best;
     return configure(b, best.first, best.second);
 }
 
@@ -459,12 +462,12 @@ int lbm_batch_info(const lbm_batch *b, int *threads, int *ctas, long long *round
 
 int lbm_batch_set_threads(lbm_batch *b, int threads)
 {
-    if (!b || (threads != 128 && threads != 256 && threads != 512)) return LBM_EINVAL;
+    if (!b || (threads != 128 && threads != 256 && threads != 512 && threads != b->tuned.first)) return LBM_EINVAL;
     if (b->exec) cudaGraphExecDestroy(b->exec);
     b->exec = nullptr;
     b->graph_steps = -1;
     // the shared memory the tuner chose goes with its CTA size; small CTAs need company on their SM
-    return configure(b, threads, threads == b->threads ? b->smem_want : 0);
+    return configure(b, threads, threads == b->tuned.first ? b->tuned.second : 0);
 }
 
 int lbm_batch_destroy(lbm_batch *b)

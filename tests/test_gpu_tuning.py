@@ -44,3 +44,23 @@ def test_step_tuner_knows_the_kernel(precision, launches):
         assert n > launches, tau
         n, again = first_step(tau)
         assert n == launches and np.array_equal(tuned, again), tau
+
+
+@pytest.mark.parametrize("nc", [3, 6])
+def test_batch_returns_to_the_tuned_size(nc):
+    from paper_2306_10652_gb300 import lbmfug
+    shape = (1, 4, 200)
+    c = seeded_mixture(520 + nc, nc, 0, shape, Tfac=1.2)
+    rho = smooth_rho(520 + nc, c, shape)[:, 0]
+    with lbmfug.Batch(c["a"], c["b"], c["omega"], c["kij"], 1.0, [(c["T"], rho)] * 300) as b:
+        tuned = b.info()
+        for threads in (128, 256, 512):
+            b.set_threads(threads)
+            assert b.info()["threads"] == threads
+            b.set_threads(tuned["threads"])
+            assert {k: b.info()[k] for k in ("threads", "ctas")} == {k: tuned[k] for k in ("threads", "ctas")}
+        for threads in (64, 100, 2048):
+            with pytest.raises(lbmfug.LbmError):
+                b.set_threads(threads)
+        b.run(max_steps=10, check_every=10, tol=0.0)
+        assert np.isfinite(b.state(0)["rho"]).all()
