@@ -11,9 +11,8 @@
 //   TwoSum      s + e = a + b exactly              (Knuth, TAOCP 2, 4.2.2)
 //   FastTwoSum  s + e = a + b exactly if |a| >= |b| (Dekker 1971)
 //   TwoProd     p + e = a * b exactly, e = fma(a, b, -p)
-// Sums of products use compensated dot products (after Ogita, Rump and Oishi
-// 2005, "Dot2").  The relative error of every derived quantity is about 2^-44 (binary64: 2^-53, binary32:
-// 2^-24); the tests compare ln f_i, mu_i and the force with the binary64
+// The relative error of every derived quantity is about 2^-44 (binary64: 2^-53,
+// binary32: 2^-24); the tests compare ln f_i, mu_i and the force with the binary64
 // oracle at that level.
 #pragma once
 
@@ -94,20 +93,6 @@ __device__ __forceinline__ float rcp_approx(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-
-// Compensated sum of products sum_j c_j x_j (c_j, x_j in df64) whose products
-// c_j.hi x_j.hi are all non-negative (psi of Eq. 4).
-struct DotPos {
-    float s, c;
-    __device__ __forceinline__ void add(F2 cj, F2 xj)
-    {
-        const F2 p = two_prod(cj.hi, xj.hi);
-        const F2 t = two_sum_pos(s, p.hi);
-        s = t.hi;
-        c = __fadd_rn(c, __fadd_rn(t.lo, fmaf(cj.hi, xj.lo, fmaf(cj.lo, xj.hi, p.lo))));
-    }
-    __device__ __forceinline__ F2 value() const { return fast_two_sum(s, c); }
-};
 
 // ---- packed FP32x2 operations --------------------------------------------------
 // One instruction does the binary32 operation on both lanes, each rounded as

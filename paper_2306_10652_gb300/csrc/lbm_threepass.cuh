@@ -558,10 +558,7 @@ template <int LAT, int NC, typename S> struct Impl {
         const unsigned G = blocks_for(P.N, T);
         const size_t sm = (size_t)NC * Lattice<LAT>::D * T * sizeof(double);
         auto collide = P.omega == 1.0 ? k_collide<LAT, S, true, true> : k_collide<LAT, S, true, false>;
-        if (sm > 48 * 1024 &&
-            cudaFuncSetAttribute(collide, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(kMaxNc * Lattice<LAT>::D * 128 * sizeof(double))) != cudaSuccess)
-            return (int)cudaGetLastError();
+        static_assert(kMaxNc * 3 * 128 * sizeof(double) <= 48 * 1024, "the forces fit the default limit");
         k_sums<LAT, S, true><<<G, T, 0, s>>>(w.par, in, w.rho, w.psi, w.jm);
         k_eos<LAT, NC, true><<<G, T, 0, s>>>(w.par, w.rho, w.psi, w.lnf, nullptr, nullptr);
         collide<<<G, T, sm, s>>>(w.par, in, out, w.rho, w.lnf, nullptr, w.jm, nullptr, w.osum, w.ocmp);
