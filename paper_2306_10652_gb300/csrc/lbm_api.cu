@@ -440,11 +440,17 @@ int ensure_allocated(lbm_problem *p)
     }
     const size_t fb = nf * sizeof(double);
     p->w.rho = (double *)dev_alloc(p, fb);
-    p->w.lnf = (double *)dev_alloc(p, fb);
-    p->mu = (float2 *)p->w.lnf;  // LBM_FP32DEV: both live within one step or one call only
-    p->w.psi = (double *)dev_alloc(p, (size_t)p->N * sizeof(double));
-    p->w.lap = (double *)dev_alloc(p, (size_t)p->N * sizeof(double));
-    p->w.jm = (double *)dev_alloc(p, (size_t)p->D * p->N * sizeof(double));
+    // ln f, psi and lap psi in one block: what lives in them lives within one step or one
+    // call, so the mu of an LBM_FP32DEV step and a host velocity on its way in use it too
+    p->w.lnf = (double *)dev_alloc(p, fb + 2 * (size_t)p->N * sizeof(double));
+    if (!p->w.rho || !p->w.lnf) return LBM_ENOMEM;
+    p->mu = (float2 *)p->w.lnf;
+    p->w.psi = p->w.lnf + nf;
+    p->w.lap = p->w.psi + p->N;
+    if (!p->fused && !p->multipass && !p->resident) {
+        p->w.jm = (double *)dev_alloc(p, (size_t)p->D * p->N * sizeof(double));
+        if (!p->w.jm) return LBM_ENOMEM;
+    }
     Log64 *lt = (Log64 *)dev_alloc(p, sizeof(Log64));
     if (!lt) return LBM_ENOMEM;
     if (cudaMemcpyAsync(lt, &log64_host(), sizeof(Log64), cudaMemcpyHostToDevice, p->stream) != cudaSuccess)
@@ -479,9 +485,7 @@ int ensure_allocated(lbm_problem *p)
     p->res = (double *)dev_alloc(p, 64 * sizeof(double));
     p->flag = (int *)dev_alloc(p, 16);
     p->mon = (double *)dev_alloc(p, kMaxNc * sizeof(double));
-    if (!p->mon || !p->w.rho || !p->w.lnf || !p->w.psi || !p->w.lap || !p->w.jm ||
-        !p->partials || !p->res || !p->flag)
-        return LBM_ENOMEM;
+    if (!p->mon || !p->partials || !p->res || !p->flag) return LBM_ENOMEM;
     if (p->fused) {
         p->nsm = nsm;
         size_t parts = 0;
@@ -950,14 +954,15 @@ int lbm_init_fields(lbm_problem *p, const double *rho, const double *u)
     if (u && !all_finite(u, (size_t)p->D * p->N)) return LBM_EINVAL;
     int st = ensure_allocated(p);
     if (st) return st;
-    // stage through the three-pass scratch (rho: nc*N doubles; u: lnf buffer holds D*N <= nc*N? no)
+    // stage through the scratch fields: rho, and u in the block of ln f, psi and lap psi (at
+    // least 3 N values)
     double *d_rho = p->w.rho;
     double *d_u = nullptr;
     if (cudaMemcpyAsync(d_rho, rho, nrho * sizeof(double), cudaMemcpyHostToDevice, p->stream) !=
         cudaSuccess)
         return LBM_ECUDA;
     if (u) {
-        d_u = p->w.jm;  // D*N doubles
+        d_u = p->w.lnf;
         if (cudaMemcpyAsync(d_u, u, (size_t)p->D * p->N * sizeof(double), cudaMemcpyHostToDevice,
                             p->stream) != cudaSuccess)
             return LBM_ECUDA;

@@ -158,10 +158,10 @@ __device__ __forceinline__ void store_pair(void *base, bool one, int p, long lon
 // Scratch fields of the three-pass schedule (device).
 struct ThreePassWork {
     double *rho;  // [nc][N] mass densities rho_i
-    double *lnf;  // [nc][N] ln f_i (the step: mu_i / (M_i RT))
+    double *lnf;  // [nc][N] ln f_i (the step: mu_i / (M_i RT)); followed by psi and lap
     double *psi;  // [N]     psi = sum_j sqrt(kappa_j) rho~_j
     double *lap;  // [N]     lap psi
-    double *jm;   // [D][N]  sum_i sum_a e_a g_{a,i}
+    double *jm;   // [D][N]  sum_i sum_a e_a g_{a,i} (of a step: null in the other schedules)
     Par64 par;              // constants of the binary64 passes (its table is on the device)
     float *osum;  // [nc][N] binary32 storage: compensated sum of the populations
     float *ocmp;  //         that left each node in the last collision

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kThreads)
     }
 }
 
-// Densities, and for kFull the momentum and psi.  kFull = false (only the
+// Densities, and for kFull psi and the momentum (jm may be null).  kFull = false (only the
 // densities are asked for): binary32 storage reads its pairs and no population.
 template <int LAT, typename S, bool kFull>
 __global__ void __launch_bounds__(kThreads)
@@ -234,6 +234,7 @@ __global__ void __launch_bounds__(kThreads)
     }
     if constexpr (kFull) {
         psi[r] = ps;
+        if (!jm) return;
         if constexpr (sizeof(S) == 8) {
             double j[3] = {0.0, 0.0, 0.0};
 #pragma unroll
@@ -319,7 +320,7 @@ template <int LAT, typename S, bool STEP, bool TAU1>
 __global__ void __launch_bounds__(kThreads)
     k_collide(const Par64 P, StateBufs in, StateBufs out, const double *__restrict__ rho,
               const double *__restrict__ X, const double *__restrict__ lap,
-              const double *__restrict__ jm, double *__restrict__ uout, float *__restrict__ osum,
+              const double *jm, double *uout /* may be jm */, float *__restrict__ osum,
               float *__restrict__ ocmp)
 {
     using L = Lattice<LAT>;
@@ -373,7 +374,7 @@ __global__ void __launch_bounds__(kThreads)
     const double irt = rcp64(rt), cs = 0.5 / (3.0 * sf);
     double u[D];
 #pragma unroll
-    for (int d = 0; d < D; ++d) u[d] = fma(cs, Fs[d], __ldg(jm + d * N + r)) * irt;
+    for (int d = 0; d < D; ++d) u[d] = fma(cs, Fs[d], jm[d * N + r]) * irt;
     if constexpr (!STEP) {
 #pragma unroll
         for (int d = 0; d < D; ++d) uout[d * N + r] = u[d];
@@ -579,11 +580,12 @@ template <int LAT, int NC, typename S> struct Impl {
             return (int)cudaGetLastError();
         }
         double *lf = lnf ? lnf : (u ? w.lnf : nullptr);
-        k_sums<LAT, S, true><<<G, T, 0, s>>>(w.par, st, r, w.psi, w.jm);
+        // (the momentum of a node waits in the place of its velocity)
+        k_sums<LAT, S, true><<<G, T, 0, s>>>(w.par, st, r, w.psi, u);
         k_eos<LAT, NC, false><<<G, T, 0, s>>>(w.par, r, w.psi, lf, p, u ? w.lap : nullptr);
         if (u)
             k_collide<LAT, S, false, false>
-                <<<G, T, 0, s>>>(w.par, st, StateBufs{}, r, lf, w.lap, w.jm, u, nullptr, nullptr);
+                <<<G, T, 0, s>>>(w.par, st, StateBufs{}, r, lf, w.lap, u, u, nullptr, nullptr);
         return (int)cudaGetLastError();
     }
     static int to_f64(const Params &P, StateBufs st, double *out, cudaStream_t s)
