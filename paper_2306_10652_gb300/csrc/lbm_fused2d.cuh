@@ -343,9 +343,11 @@ struct Par32 {
     int nx, ny;
     long long N;
     float om1;           // 1 - w
-    float so3, sg, cs;   // 3 w / 36; (1 - w/2)/432; F/2 from f: 0.5 * 36 / (3 (1 - w/2))
+    float2 so3;          // 3 w / 36 in two words: one is off by up to 2^-25, the same in every
+                         // node and step, and so would be the momentum that a step hands on
+    float sg, cs;        // (1 - w/2)/432; F/2 from f: 0.5 * 36 / (3 (1 - w/2))
     float RT, lnRT;
-    float2 cf[kMaxNc / 2];   // f_i / (rho_i X), X = grad mu_i (double-binary32) or 12 grad mu_i
+    float2 cf[kMaxNc / 2], cfl[kMaxNc / 2];  // f_i / (rho_i X), X = grad mu_i (double-binary32) or 12 grad mu_i: two words
     float invM[kMaxNc], sqk[kMaxNc], b[kMaxNc], A[kMaxNc * kMaxNc];
 };
 
@@ -357,14 +359,16 @@ inline Par32 make_par32(const Params &P, bool df)
     q.ny = P.ny;
     q.N = P.N;
     q.om1 = (float)(1.0 - P.omega);
-    q.so3 = (float)(P.omega / 12.0);
+    q.so3.x = (float)(P.omega / 12.0);
+    q.so3.y = (float)(P.omega / 12.0 - (double)q.so3.x);
     q.sg = (float)(cF / 432.0);
     q.cs = (float)(6.0 / cF);
     q.RT = P.fRT;
     q.lnRT = P.flnRT;
     for (int i = 0; i < P.nc; ++i) {
-        const float c = (float)(-cF / (df ? 12.0 : 144.0) * P.invM[i]);
-        (i & 1 ? q.cf[i / 2].y : q.cf[i / 2].x) = c;
+        const double c = -cF / (df ? 12.0 : 144.0) * P.invM[i];
+        (i & 1 ? q.cf[i / 2].y : q.cf[i / 2].x) = (float)c;
+        (i & 1 ? q.cfl[i / 2].y : q.cfl[i / 2].x) = (float)(c - (double)(float)c);
         q.invM[i] = P.finvM[i];
         q.sqk[i] = P.fsqk[i];
         q.b[i] = P.fb[i];
@@ -774,7 +778,7 @@ __global__ void __launch_bounds__(kT, NC == 1 ? 6 : NC <= 6 ? 4 : NC <= 10 ? 3 :
             for (int p = 0; p < NP; ++p) {
                 const float2 ri = R1[p * kT];
                 rs = vadd(rs, ri);
-                const float2 cr = vmul(P.cf[p], ri);
+                const float2 cr = vfma(P.cf[p], ri, vmul(P.cfl[p], ri));
                 float2 gx, gy;
                 if constexpr (kDF) {
                     if (one(p)) {
@@ -797,7 +801,7 @@ __global__ void __launch_bounds__(kT, NC == 1 ? 6 : NC <= 6 ? 4 : NC <= 10 ? 3 :
                 Fsy = vadd(Fsy, fy[p]);
             }
             const float rt = rs.x + rs.y, Fx = Fsx.x + Fsx.y, Fy = Fsy.x + Fsy.y;
-            const float irt = __fdividef(1.0f, rt);
+            const float irt = rcp32(rt);
             const float u0 = fmaf(P.cs, Fx, jq.x) * irt;
             const float u1 = fmaf(P.cs, Fy, jq.y) * irt;
             const float h2 = -0.5f * fmaf(u0, u0, u1 * u1);
@@ -825,7 +829,7 @@ __global__ void __launch_bounds__(kT, NC == 1 ? 6 : NC <= 6 ? 4 : NC <= 10 ? 3 :
                     Gsx = vadd(Gsx, Gx);
                     Gsy = vadd(Gsy, Gy);
                 }
-                const float2 r3 = vmul(vbc(P.so3), R1[p * kT]);
+                const float2 r3 = vfma(vbc(P.so3.x), R1[p * kT], vmul(vbc(P.so3.y), R1[p * kT]));
                 const float2 Vx = vfma(r3, ux, fx[p]), Vy = vfma(r3, uy, fy[p]);
                 const float2 sg3 = vbc(3.0f * P.sg);
                 const float2 Hx = vfma(sg3, Gx, vmul(vbc(1.5f), vadd(Vx, fx[p])));
@@ -874,7 +878,7 @@ __global__ void __launch_bounds__(kT, NC == 1 ? 6 : NC <= 6 ? 4 : NC <= 10 ? 3 :
             }
             float s[9];  // collided values summed over the components
             if constexpr (TAU1) {
-                const float Gx = Gsx.x + Gsx.y, Gy = Gsy.x + Gsy.y, r3 = P.so3 * rt;
+                const float Gx = Gsx.x + Gsx.y, Gy = Gsy.x + Gsy.y, r3 = fmaf(P.so3.x, rt, P.so3.y * rt);
                 const float Vx = fmaf(r3, u0, Fx), Vy = fmaf(r3, u1, Fy);
                 const float Hx = fmaf(3.0f * P.sg, Gx, 1.5f * (Vx + Fx)), Hy = fmaf(3.0f * P.sg, Gy, 1.5f * (Vy + Fy));
                 const float fu = fmaf(Fx, u0, Fy * u1), gu = P.sg * fmaf(Gx, u0, Gy * u1);

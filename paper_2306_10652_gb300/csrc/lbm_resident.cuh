@@ -260,7 +260,11 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const Par P, StateBufs st,
     R *psi = (R *)W.psi;
     S *gx = (S *)W.g + i;  // [8][N][G]
     const S om = TAU1 ? (S)1 : (S)P.omega, om1 = (S)1 - om;
-    const S sf = (S)((1.0 - 0.5 * (TAU1 ? 1.0 : P.omega)) / 36.0), sg = sf / (S)12, so3 = om / (S)12;
+    const S sf = (S)((1.0 - 0.5 * (TAU1 ? 1.0 : P.omega)) / 36.0), sg = sf / (S)12;
+    // w/12 in two words in binary32: one is off by up to 2^-25, the same in every step, and so
+    // would be the momentum that a step hands on
+    const double w12 = (TAU1 ? 1.0 : P.omega) / 12.0;
+    const S so3 = (S)w12, so3l = k64 ? (S)0 : (S)(w12 - (double)so3);
     const S cs = (S)0.5 / ((S)3 * sf);
     // f_i from 12 grad(mu): mu / (M RT) for binary32 and binary64, mu for double-binary32
     const S cf = kDF ? (S)(-0.25) * sf * (S)(on ? P.p64->invM[i] : 0.0) : (S)(-0.25 * P.RT) * sf;
@@ -320,11 +324,13 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const Par P, StateBufs st,
             Gy = fma((S)4, q[3], q[5] - q[7]);
         }
         const S Fx = bfly<G>(fx), Fy = bfly<G>(fy);
-        const S irt = lane_rcp(rt);
+        S irt;
+        if constexpr (k64) irt = rcp64(rt);
+        else irt = rcp32(rt);
         const S ux = fma(cs, Fx, jx) * irt, uy = fma(cs, Fy, jy) * irt;
         if (on) {
             const S hu2 = (S)(-0.5) * fma(ux, ux, uy * uy);
-            const S r3 = so3 * r;
+            const S r3 = k64 ? so3 * r : fma(so3, r, so3l * r);
             const S Vx = fma(r3, ux, fx), Vy = fma(r3, uy, fy);
             const S Hx = fma((S)3 * sg, Gx, (S)1.5 * (Vx + fx)), Hy = fma((S)3 * sg, Gy, (S)1.5 * (Vy + fy));
             const S fu = fma(fx, ux, fy * uy), gu = sg * fma(Gx, ux, Gy * uy);
