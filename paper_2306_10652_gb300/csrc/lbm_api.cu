@@ -353,6 +353,7 @@ void build_par64(lbm_problem *p, const Log64 *tab)
     q.c2 = c2.hi;
     q.c2l = c2.lo;
     const D2 lnRT = dd_log(P.RT);
+    q.lnRTl = lnRT.lo;
     q.omega = P.omega;
     q.tab = tab;
     for (int i = 0; i < P.nc; ++i) {
@@ -363,9 +364,7 @@ void build_par64(lbm_problem *p, const Log64 *tab)
         q.bM[i] = P.b[i] * P.invM[i];
         q.pk[i] = P.sqk[i] * P.invM[i];
         q.kM[i] = q.pk[i] / P.RT;
-        const D2 c0 = dd_add(lnRT, dd_log(P.invM[i]));
-        q.c0[i] = c0.hi;
-        q.c0l[i] = c0.lo;
+        q.c0[i] = dd_add({lnRT.hi, 0.0}, dd_log(P.invM[i])).hi;
         for (int j = 0; j < P.nc; ++j) q.A[i * kMaxNc + j] = P.A[i * kMaxNc + j] * P.invM[i] * P.invM[j];
     }
 }

@@ -120,7 +120,10 @@ template <int G, typename E> struct Thermo {
         const E Q = bfly<G>(r * T);
         const E omB = (E)1 - B, den = fma(B, (E)2 - B, (E)1);
         const E u = lane_rcp(B), vb = lane_rcp(omB), vd = lane_rcp(den);
-        const E Lu = lane_log(fma((E)1 + kS2, B, (E)1) * lane_rcp(fma((E)1 - kS2, B, (E)1)), tab) * u;
+        const E n1 = fma((E)1 + kS2, B, (E)1), n2 = fma((E)1 - kS2, B, (E)1), w = n1 * vd;
+        E q = n1 * w;
+        q = fma(fma(-q, n2, n1), w, q);
+        const E Lu = lane_log(q, tab) * u;
         const E C0 = -lane_log(omB, tab);
         const E qu = Q * u;
         E iRT, iRTl, c2, c2l;

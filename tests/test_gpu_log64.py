@@ -4,8 +4,8 @@ precision, beside CUDA's log and division on the same arguments.
 Bounds.  log64: the last addition rounds once (half an ulp of the result); before it,
 |r^5 - 0.87 2^-22 r^3| / 5 <= 0.13 2^-55 / 5 of the polynomial, r^6 / 6 <= 2^-68, one
 rounding of a sum below 2^-11 (2^-65) and the low words of the tables (2^-67 each):
-8e-19 together.  rcp64: the seed is good to 2^-20, so two Newton steps leave 2^-80
-before the last operation, which rounds once: half an ulp and 2^-20 of one.
+8e-19 together.  rcp64: the seed is good to 2^-20, so the series cut after the square
+leaves 2^-60 before the last operation, which rounds once: half an ulp and 2^-6 of one.
 """
 from __future__ import annotations
 
@@ -87,16 +87,22 @@ def test_rcp64_rounds_once(evaluate, lo, hi):
     got = evaluate(np.concatenate([x, -x]))[2]
     ref = np.longdouble(1) / np.concatenate([x, -x]).astype(np.longdouble)
     e = np.abs(got - ref).astype(np.float64)
-    assert (e <= (0.5 + 2.0**-20) * np.spacing(np.abs(got))).all()
+    assert (e <= (0.5 + 2.0**-6) * np.spacing(np.abs(got))).all()
 
 
-def test_special_arguments_take_the_library(evaluate):
-    tiny = np.finfo(np.float64).tiny
-    x = np.array([0.0, -0.0, np.inf, -np.inf, np.nan, -1.0, 5e-324, tiny / 3, tiny, -tiny, np.finfo(np.float64).max,
-                  2.0**1021, 2.0**1022, 2.0**1023, 1.0, 0.5, 2.0])
-    l, lc, r, rc = evaluate(x)
-    assert np.array_equal(r, rc, equal_nan=True)
-    assert np.array_equal(l[:8], lc[:8], equal_nan=True)
-    assert abs(l[14]) <= 8e-19  # ln 1: the part before the last addition
-    # the powers of two: multiples of ln 2, rounded once
-    assert np.array_equal(l[15:], lc[15:])
+def test_special_arguments(evaluate):
+    tiny, big = np.finfo(np.float64).tiny, np.finfo(np.float64).max
+    # zeros, infinities, NaN and exact reciprocals as the division gives them
+    x = np.array([0.0, -0.0, np.inf, -np.inf, np.nan, 1.0, -1.0, 0.5, -2.0, tiny, -tiny, 2.0**1021, 2.0**1022])
+    _, _, r, rc = evaluate(x)
+    assert np.array_equal(r, rc, equal_nan=True) and np.array_equal(np.signbit(r), np.signbit(rc))
+    # subnormal arguments count as zeros, subnormal results may be
+    assert np.array_equal(evaluate([5e-324, tiny / 3, -tiny / 3])[2], [np.inf, np.inf, -np.inf])
+    assert (np.abs(evaluate([big, -big, 2.0**1023])[2]) < tiny).all()
+    # log64: the library's log where the table does not reach, and ln 1 to the part before the
+    # last addition
+    x = np.array([0.0, -0.0, np.inf, -np.inf, np.nan, -1.0, 5e-324, tiny / 3])
+    l, lc, _, _ = evaluate(x)
+    assert np.array_equal(l, lc, equal_nan=True)
+    l, lc, _, _ = evaluate([1.0, 0.5, 2.0, 1024.0])
+    assert abs(l[0]) <= 8e-19 and np.array_equal(l[1:], lc[1:])
