@@ -288,9 +288,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const Par P, StateBufs st,
     // density (binary64), momentum, psi and total density of a state
     auto close = [&]() {
         if constexpr (k64) {
-            r = v[0];
+            r = v[1];  // (the resting one last, see k_sums)
 #pragma unroll
-            for (int a = 1; a < 9; ++a) r += v[a];
+            for (int a = 2; a < 9; ++a) r += v[a];
+            r = v[0] + r;
         }
         jx = bfly<G>((v[1] - v[2]) + (v[5] - v[6]) + (v[7] - v[8]));
         jy = bfly<G>((v[3] - v[4]) + (v[5] - v[6]) + (v[8] - v[7]));

@@ -207,9 +207,12 @@ __global__ void __launch_bounds__(kThreads)
         }
         double ri;
         if constexpr (sizeof(S) == 8) {
-            ri = v[0];
+            // the moving populations first: they are small beside the resting one, which
+            // carries the density, so one addition rounds at its size instead of Q - 1
+            double m = v[1];
 #pragma unroll
-            for (int a = 1; a < L::Q; ++a) ri += v[a];
+            for (int a = 2; a < L::Q; ++a) m += v[a];
+            ri = v[0] + m;
         } else {
             ri = widen(__ldg(rh + st.at(i, N, r))) + widen(__ldg(rl + st.at(i, N, r)));
         }

@@ -8,13 +8,15 @@ steps sees.
   wave of this length by far less than itself) and to random roundings: bound 1e-8 a step.
 * Batched jobs start at rest: a standing density wave, half of whose energy is motion, so
   half of the bound.
+* Density of a binary64 state: the moving populations are added first, so the sum is off by
+  half an ulp of the density and the roundings of sums of the moving populations.
 """
 from __future__ import annotations
 
 import numpy as np
 import pytest
 
-from helpers import gpu_problem, seeded_mixture
+from helpers import gpu_problem, seeded_mixture, smooth_rho
 
 pytestmark = pytest.mark.gpu
 
@@ -73,3 +75,21 @@ def test_amplitude_of_a_batched_density_wave(tau):
             ref = (gp.moments(want=("rho",))["rho"] * wave).sum(axis=(1, 2, 3))
             got = (bt.state(0)["rho"][:, None] * wave).sum(axis=(1, 2, 3))
             assert (np.abs(got - ref) <= 0.5e-8 * done * start).all(), (done, (got - ref) / start)
+
+
+@pytest.mark.parametrize("schedule,lattice,shape", [(AUTO, 0, (1, 8, 21)), (THREEPASS, 0, (1, 20, 33)),
+                                                    (THREEPASS, 1, (5, 6, 7))], ids=["resident", "d2q9", "d3q19"])
+def test_binary64_density_rounds_once(schedule, lattice, shape):
+    nc = 3
+    c = seeded_mixture(560, nc, lattice, shape, Tfac=1.2)
+    rho = smooth_rho(560, c, shape)
+    with gpu_problem(c, lattice, shape, schedule=schedule) as gp:
+        gp.init_fields(rho)
+        gp.step(5)
+        g = gp.get_state()
+        got = gp.moments(want=("rho",))["rho"]
+    ref = g.astype(np.longdouble).sum(axis=1)
+    moving = np.abs(g[:, 1:]).sum(axis=1)
+    bound = 0.5 * np.spacing(np.abs(got)) + (g.shape[1] - 2) * 0.5 * np.spacing(moving)
+    assert (np.abs(got - ref) <= bound).all()
+    assert (bound < np.spacing(np.abs(got))).mean() > 0.5  # the case is met: small moving populations
