@@ -79,7 +79,10 @@ template <int G> __device__ __forceinline__ float bfly_max(float v)
     return v;
 }
 
-__device__ __forceinline__ float lane_log(float x, const Log64 *) { return __logf(x); }
+// (binary32: the chain of a step hides most of logf, and __logf, whose absolute error is
+// 2^-21.4, is the largest rounding of mu: 400 x 2, Nc = 10, 200 steps, error of the
+// densities 5.3e-8 with logf, 1.1e-7 with __logf, at 6.4 and 6.2 us per step)
+__device__ __forceinline__ float lane_log(float x, const Log64 *) { return logf(x); }
 __device__ __forceinline__ double lane_log(double x, const Log64 *t) { return log64(x, t); }
 __device__ __forceinline__ float lane_rcp(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ double lane_rcp(double x) { return rcp64(x); }

@@ -10,13 +10,14 @@ steps sees.
   half of the bound.
 * Density of a binary64 state: the moving populations are added first, so the sum is off by
   half an ulp of the density and the roundings of sums of the moving populations.
+* LBM_FP32: the resident schedule is as accurate as the fused one.
 """
 from __future__ import annotations
 
 import numpy as np
 import pytest
 
-from helpers import gpu_problem, seeded_mixture, smooth_rho
+from helpers import gpu_problem, oracle_problem, seeded_mixture, smooth_rho
 
 pytestmark = pytest.mark.gpu
 
@@ -93,3 +94,19 @@ def test_binary64_density_rounds_once(schedule, lattice, shape):
     bound = 0.5 * np.spacing(np.abs(got)) + (g.shape[1] - 2) * 0.5 * np.spacing(moving)
     assert (np.abs(got - ref) <= bound).all()
     assert (bound < np.spacing(np.abs(got))).mean() > 0.5  # the case is met: small moving populations
+
+
+@pytest.mark.parametrize("nc,seed", [(2, 571), (4, 572), (8, 573)])
+def test_resident_binary32_is_as_accurate_as_fused(nc, seed):
+    shape, steps = (1, 4, 128), 200
+    c = seeded_mixture(seed, nc, 0, shape, Tfac=1.2)
+    rho = smooth_rho(seed, c, shape)
+    orc = oracle_problem(c, 0, shape)
+    ref = orc.step(orc.init_equilibrium(rho), steps).sum(axis=1)
+    err = {}
+    for schedule in (AUTO, FUSED):
+        with gpu_problem(c, 0, shape, precision=FP32, schedule=schedule, tune=0) as gp:
+            gp.init_fields(rho)
+            gp.step(steps)
+            err[schedule] = np.sqrt(((gp.moments(want=("rho",))["rho"] - ref) ** 2).mean())
+    assert err[AUTO] <= 1.25 * err[FUSED], err
