@@ -129,7 +129,7 @@ bool fused_supported(int lat, int prec, int nc)
 {
     if (lat != 0) return false;
     const fz::Ops *o = lookup(prec, nc);
-    return o && o->smem(o->wmax) <= max_optin_smem();
+    return o && o->smem(false, o->wmax) <= max_optin_smem();
 }
 
 // Launch geometry: strips of at most wmax columns (extra_strips more than the
@@ -146,7 +146,7 @@ FusedGeom fused_geometry(int prec, int nc, const Params &P, int num_sms, int ext
     if (g.nstrips > P.nx) g.nstrips = P.nx;
     g.strip = (P.nx + g.nstrips - 1) / g.nstrips;   // balanced strip width <= wmax
     g.nstrips = (P.nx + g.strip - 1) / g.strip;
-    g.smem = o->smem(g.strip);
+    g.smem = o->smem(P.omega == 1.0, g.strip);
     int per_sm = o->occupancy(P.omega == 1.0, g.smem);
     if (per_sm < 1) per_sm = 1;
     const long long slots = (long long)num_sms * per_sm * (seg_mult > 0 ? seg_mult : 1);
@@ -179,7 +179,7 @@ FusedGeom fused_geometry_forced(int prec, int nc, const Params &P, int num_sms, 
         g.strip = strip < o->wmax ? strip : o->wmax;
         if (g.strip > P.nx) g.strip = P.nx;
         g.nstrips = (P.nx + g.strip - 1) / g.strip;
-        g.smem = o->smem(g.strip);
+        g.smem = o->smem(P.omega == 1.0, g.strip);
     }
     if (seg_h > 0) {
         g.seg_h = seg_h < P.ny ? seg_h : P.ny;

@@ -403,7 +403,23 @@ template <int NC, typename E> struct Smem32 {
     static __host__ __device__ constexpr size_t j() { return (size_t)kT * sizeof(float2); }
     static __host__ __device__ constexpr size_t xj() { return (size_t)6 * kT * sizeof(float); }
     static __host__ __device__ constexpr size_t ps() { return kDF ? 0 : (size_t)3 * kT * sizeof(float); }
-    static __host__ __device__ constexpr size_t total() { return rs() + g() + mu() + xc() + j() + xj() + ps(); }
+    // CTAs per SM that the registers are cut for.  At general tau the largest odd number of
+    // components of a class, whose last pair has addresses of its own, waits less with one
+    // CTA fewer and no spilled registers (2048 x 1024, tau = 0.8, LBM_FP32: Nc = 5 212 us,
+    // 223 with four; Nc = 9 408 us, 447 with three; Nc = 7 304 us, 340 with two).
+    static __host__ __device__ constexpr int ctas(bool tau1)
+    {
+        const bool odd = !tau1 && (NC == 5 || NC == 9);
+        return NC == 1 ? 6 : NC <= 6 ? (odd ? 3 : 4) : NC <= 10 ? (odd ? 2 : 3) : 2;
+    }
+    // General tau: the old populations of the next pair are copied ahead of it.  More
+    // pairs than two hide their loads behind each other, and lose registers by it (same
+    // box, with and without: LBM_FP32 Nc = 2 86 and 99 us, Nc = 3 130 and 138, Nc = 6
+    // 254 and 213, Nc = 8 331 and 297).
+    static __host__ __device__ constexpr bool ahead(bool tau1) { return !tau1 && NC <= 4; }
+    static __host__ __device__ constexpr size_t v() { return (size_t)8 * kT * sizeof(float2); }
+    static __host__ __device__ constexpr size_t base() { return rs() + g() + mu() + xc() + j() + xj() + ps(); }
+    static __host__ __device__ constexpr size_t total(bool tau1) { return base() + (ahead(tau1) ? v() : 0); }
 };
 // *a = x where `on` (a predicated store, no branch)
 __device__ __forceinline__ void store_if(bool on, float2 *a, float2 x)
@@ -477,7 +493,7 @@ template <int NC> struct SmemMu {
 };
 
 template <int NC>
-__global__ void __launch_bounds__(kT, NC <= 10 ? 4 : 3)
+__global__ void __launch_bounds__(kT, NC <= 10 && NC != 9 ? 4 : 3)
     k_mu32(const df::ParMu P, const int W, const int H, StateBufs in, float4 *__restrict__ G)
 {
     constexpr int NP = SmemMu<NC>::NP, CW = NP * kT;
@@ -611,17 +627,20 @@ __global__ void __launch_bounds__(kT, NC <= 10 ? 4 : 3)
 // per SM, 0.134 ms with three, 0.141 ms with three and the components apart, 0.260 ms
 // at first; Nc = 10 needs more than the 128 registers that four leave it.
 template <int NC, typename E, bool TAU1>
-__global__ void __launch_bounds__(kT, NC == 1 ? 6 : NC <= 6 ? 4 : NC <= 10 ? 3 : 2)
+__global__ void __launch_bounds__(kT, (Smem32<NC, E>::ctas(TAU1)))
     k_fused32(const Par32 P, const int W, const int H, StateBufs in, StateBufs out,
               const float4 *__restrict__ mug /* DF64: grad mu of a pair of components (x, x, y, y); an odd last one (x, y) */)
 {
     using L = Lattice<0>;
     using SM = Smem32<NC, E>;
-    using df::vadd;
     using df::vbc;
-    using df::vfma;
-    using df::vmul;
-    constexpr bool kDF = SM::kDF;
+    // one component alone: the other lane stays zero and costs nothing
+    auto vadd = [](float2 a, float2 b) { return NC == 1 ? make_float2(__fadd_rn(a.x, b.x), 0.0f) : df::vadd(a, b); };
+    auto vmul = [](float2 a, float2 b) { return NC == 1 ? make_float2(__fmul_rn(a.x, b.x), 0.0f) : df::vmul(a, b); };
+    auto vfma = [](float2 a, float2 b, float2 c) {
+        return NC == 1 ? make_float2(__fmaf_rn(a.x, b.x, c.x), 0.0f) : df::vfma(a, b, c);
+    };
+    constexpr bool kDF = SM::kDF, AHEAD = SM::ahead(TAU1);
     constexpr int NP = SM::NP, kHalo = SM::kHalo, kRing = SM::kRing, kLag = kDF ? 1 : 2;
     constexpr int CW = NP * kT;  // a ring slot
     auto one = [](int p) { return 2 * p + 1 == NC; };  // an odd last component
@@ -631,7 +650,8 @@ __global__ void __launch_bounds__(kT, NC == 1 ? 6 : NC <= 6 ? 4 : NC <= 10 ? 3 :
     float2 *MU = (float2 *)((unsigned char *)GS + SM::g());   // [3][NP][kT] mu rows (binary32)
     float2 *XC = (float2 *)((unsigned char *)MU + SM::mu());  // [6][NP][kT] exchange
     float2 *JS = XC + 6 * CW;                                 // [kT] momentum of row q
-    float *XJ = (float *)(JS + kT);                           // [6][kT]
+    float2 *VS = JS + kT;                                     // [8][kT] AHEAD: old populations of a pair
+    float *XJ = (float *)(VS + (AHEAD ? 8 * kT : 0));         // [6][kT]
     float *PS = XJ + 6 * kT;                                  // [3][kT] psi rows (binary32)
     const void *__restrict__ gin = in.g;
     void *__restrict__ gout = out.g;
@@ -688,6 +708,15 @@ __global__ void __launch_bounds__(kT, NC == 1 ? 6 : NC <= 6 ? 4 : NC <= 10 ? 3 :
                 if (one(p)) copy_async<8>(GS + p * kT + t, (const float2 *)(mug + p * N) + o);
                 else copy_async<16>(GS + p * kT + t, mug + p * N + o);
             }
+        }
+    };
+
+    // the old populations of a pair, one pair ahead of its collision
+    auto copy_populations = [&](int p, unsigned o) {
+#pragma unroll
+        for (int a = 0; a < 8; ++a) {
+            if (one(p)) copy_async<4>(VS + a * kT + t, (const float *)gin + (16LL * p + a) * N + o);
+            else copy_async<8>(VS + a * kT + t, (const float2 *)gin + (8LL * p + a) * N + o);
         }
     };
 
@@ -811,7 +840,7 @@ __global__ void __launch_bounds__(kT, NC == 1 ? 6 : NC <= 6 ? 4 : NC <= 10 ? 3 :
             const unsigned rq = row(crow), rn = row(crow + 1), rsn = row(crow - 1);
             const unsigned rc = rq + xg;
             const unsigned dst[9] = {rc, rq + xr, rq + xl, rn + xg, rsn + xg, rn + xr, rsn + xl, rsn + xr, rn + xl};
-            float2 S[TAU1 ? 1 : 9];  // general tau: collided values summed over the components
+            float2 S[TAU1 && NC > 1 ? 1 : 9];  // general tau, one component: collided values summed over the components
             float2 Gsx = vbc(0.0f), Gsy = vbc(0.0f);  // tau = 1: sum of 12 grad rho
             if constexpr (!TAU1)
 #pragma unroll
@@ -819,9 +848,19 @@ __global__ void __launch_bounds__(kT, NC == 1 ? 6 : NC <= 6 ? 4 : NC <= 10 ? 3 :
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
                 float2 v[9];
-                if constexpr (!TAU1) {
+                if constexpr (!TAU1 && !AHEAD) {
 #pragma unroll
                     for (int a = 1; a < 9; ++a) v[a] = load_pair(gin, one(p), p, a - 1, 8, N, rc);
+                }
+                if constexpr (AHEAD) {
+                    if (p > 0) copy_async_wait();
+#pragma unroll
+                    for (int a = 1; a < 9; ++a) {
+                        v[a] = VS[(a - 1) * kT + t];
+                        if (one(p)) v[a].y = 0.0f;
+                    }
+                    if (p + 1 < NP) copy_populations(p + 1, rc);
+                    else if (kk + 1 < nrows) copy_populations(0, rn + xg);  // of the next row
                 }
                 float2 Gx, Gy;
                 grad12(R0 + p * kT, R1 + p * kT, R2 + p * kT, Gx, Gy);
@@ -841,10 +880,9 @@ __global__ void __launch_bounds__(kT, NC == 1 ? 6 : NC <= 6 ? 4 : NC <= 10 ? 3 :
                 const float2 qx = vmul(ux, Hx), qy = vmul(uy, Hy);
                 float2 *X = XC + p * kT + t;
                 auto out1 = [&](int a, float2 g) {  // population a of the pair: Eq. (1a)
-                    if constexpr (!TAU1) {
-                        g = vfma(vbc(P.om1), v[a], g);
-                        S[a] = vadd(S[a], g);
-                    }
+                    if constexpr (!TAU1) g = vfma(vbc(P.om1), v[a], g);
+                    if constexpr (NC == 1) S[a] = g;
+                    else if constexpr (!TAU1) S[a] = vadd(S[a], g);
                     store_pair_if(st, gout, one(p), p, a - 1, 8, N, dst[a], g);
                     leave(bH[p], bL[p], g);
                     const int ex = L::e(a, 0), ey = L::e(a, 1);
@@ -877,7 +915,10 @@ __global__ void __launch_bounds__(kT, NC == 1 ? 6 : NC <= 6 ? 4 : NC <= 10 ? 3 :
                 }
             }
             float s[9];  // collided values summed over the components
-            if constexpr (TAU1) {
+            if constexpr (NC == 1) {
+#pragma unroll
+                for (int a = 1; a < 9; ++a) s[a] = S[a].x;
+            } else if constexpr (TAU1) {
                 const float Gx = Gsx.x + Gsx.y, Gy = Gsy.x + Gsy.y, r3 = fmaf(P.so3.x, rt, P.so3.y * rt);
                 const float Vx = fmaf(r3, u0, Fx), Vy = fmaf(r3, u1, Fy);
                 const float Hx = fmaf(3.0f * P.sg, Gx, 1.5f * (Vx + Fx)), Hy = fmaf(3.0f * P.sg, Gy, 1.5f * (Vy + Fy));
@@ -903,6 +944,7 @@ __global__ void __launch_bounds__(kT, NC == 1 ? 6 : NC <= 6 ? 4 : NC <= 10 ? 3 :
             jn.y = s[3];
         } else if (kk == 2 * kLag - 1) {
             copy_collision(crow + 1);  // of the first row that is collided
+            if (AHEAD && active) copy_populations(0, row(crow + 1) + xg);
         }
         __syncthreads();
         if constexpr (!kDF)  // into the slot of row k-3, whose last reader was this collision
@@ -976,7 +1018,7 @@ struct Ops {
     // potentials, [nc][N] (d/dx, d/dy) (LBM_FP32DEV), else unused.  Returns the launches made through *launches.
     int (*step)(const Params &, const df::ParMu &, const FusedGeom &, StateBufs, StateBufs, double *, float2 *mu, int *launches,
                 KernelTimer *, cudaStream_t);
-    size_t (*smem)(int W);
+    size_t (*smem)(bool tau1, int W);
     int (*occupancy)(bool tau1, size_t smem);  // CTAs per SM of the step kernel that will run
     int (*occupancy_mu)();  // CTAs per SM of the mu pass (0: the form has none)
 };
@@ -1005,17 +1047,17 @@ template <int NC, typename S, typename E> struct Impl {
         }
         return (int)cudaGetLastError();
     }
-    static size_t smem(int W)
+    static size_t smem(bool tau1, int W)
     {
         if constexpr (k64) return Smem<NC, double, double>::total(W);
-        else return Smem32<NC, E>::total();
+        else return Smem32<NC, E>::total(tau1);
     }
     static int occupancy(bool tau1, size_t bytes)
     {
         // the limit is the widest strip's need, so that problems of other
         // widths launched later keep fitting under it
         if (cudaFuncSetAttribute(kernel(tau1), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem(wmax())) != cudaSuccess)
+                                 (int)smem(tau1, wmax())) != cudaSuccess)
             return 0;
         int n = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel(tau1), kT, bytes) != cudaSuccess)
