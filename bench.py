@@ -54,10 +54,10 @@ def initial_density(d, case, nx, ny, seed=2):
 # schedule, Nc) and on the kernel they were captured from; the traffic is per
 # node (strip and segment halos come from L2), so it scales with the nodes of a
 # launch.  profiles/step_kernels.md: the step kernel k_fused32<10, DF64, tau = 1>
-# moved 378.2 + 796.8 MB over 2,097,152 nodes.
+# moved 378.7 + 800.2 MB over 2,097,152 nodes.
 # A form without an entry, or whose kernel has changed since, reports null.
 NCU_TRAFFIC_B_PER_NODE = {
-    ("fp32dev", "auto", 10): ("k_fused32<10, DF64> (step kernel)", (378.249472e6 + 796.799232e6) / 2097152),
+    ("fp32dev", "auto", 10): ("k_fused32<10, DF64> (step kernel)", (378.661376e6 + 800.186624e6) / 2097152),
 }
 
 
@@ -694,8 +694,8 @@ def run_served(args, lbmfug):
             "gpu_busy_pct": busy_pct,
             "nc_node_steps_per_s": work / (t1 - t0), "slots": args.serve_slots,
             "peak_bytes": stats["peak_bytes"], "budget_bytes": stats["budget_bytes"], "rounds": stats["rounds"],
-            "precision": "fp32dev (binary32 populations; thermodynamics double-binary32: fused D2Q9, "
-                         "multi-pass D3Q19)",
+            "precision": "fp32dev (binary32 populations; thermodynamics double-binary32: resident or "
+                         "multi-pass D2Q9, multi-pass D3Q19)",
             "fp64_one_at_a_time": {"measured": True, "solves": solved64, "wall_s": w64,
                                    "solves_per_s": solved64 / w64 if w64 > 0 else None,
                                    "sample": "requests in a seeded random order, each alone to the criterion"}}
@@ -761,7 +761,7 @@ def run_served_scale(args, lbmfug):
             "queued_s": {"p50": float(np.percentile(q, 50)), "max": float(q.max())},
             "run_s": {"p50": float(np.percentile(run, 50)), "max": float(run.max())},
             "gpu_busy_pct": busy.mean(),
-            "precision": "fp32dev (multi-pass D3Q19, fused D2Q9)"}
+            "precision": "fp32dev (multi-pass D3Q19; D2Q9 1024^2 fused, or multi-pass while it fits L2)"}
 
 
 def run_reference(args):

@@ -50,8 +50,11 @@ enum lbm_lattice { LBM_D2Q9 = 0, LBM_D3Q19 = 1 };
  *               equilibrium (rho_i, 0, ..., 0) of Eq. (1b): the Q-1 moving
  *               populations in binary32, with the density rho_i itself kept
  *               exactly as a binary32 pair (hi + lo) that each step moves by
- *               compensated sums of the populations that left and arrived
- *               (component mass conserved to the rounding of the pair);
+ *               the populations that left and arrived, every one with its
+ *               rounding error (component mass conserved to the rounding of
+ *               the pair; in the fused, resident and batched kernels while no
+ *               single population exceeds the density of the node it leaves or
+ *               enters, in the others always);
  *               collision in binary32; Peng-Robinson mixture, fugacities,
  *               chemical-potential differences of the force and mass sums at
  *               binary64 accuracy: the fused schedule evaluates them in
@@ -74,7 +77,9 @@ enum lbm_precision { LBM_FP64 = 0, LBM_FP32DEV = 1, LBM_FP32 = 2 };
  *  LBM_SCHED_THREEPASS: any lattice and storage, thermodynamics and forces
  *                       in binary64.
  *  LBM_SCHED_AUTO:      on D2Q9 many steps per launch by one thread-block
- *                       cluster for boxes of a few hundred nodes; else fused
+ *                       cluster for small boxes (nodes times Nc rounded up to
+ *                       a power of two at most 16384; LBM_FP64 4096, or 8192
+ *                       from six components on); else fused
  *                       for the binary32 storages (LBM_FP32DEV: multi-pass
  *                       while the step's exchange stays in L2).  Fused for
  *                       every form when strip or seg_h is set.  Multi-pass for
@@ -305,8 +310,9 @@ int lbm_field_sums_noalloc(const double *d_field, int nc, long long n, double *d
  * is finished and skipped from then on.  Storage is the binary32 format of
  * LBM_FP32DEV/LBM_FP32 (opt->precision selects binary64 or binary32
  * thermodynamics; LBM_FP64 is taken as LBM_FP32DEV).  The CTA size is chosen
- * by timed trials on the first creation for a given (precision, Nc, largest
- * box) and cached for the process; results do not depend on it.
+ * by timed trials on the first creation for a given (precision, Nc, tau = 1 or
+ * not, largest box, jobs per SM and mean box) and cached for the process;
+ * results do not depend on it.
  * ------------------------------------------------------------------------ */
 typedef struct lbm_job {
     int nx, ny;          /* periodic box, nx * ny <= 2^20 and fitting shared memory */

@@ -393,13 +393,13 @@ int ensure_allocated(lbm_problem *p)
     // binary64 runs the three-pass schedule unless the fused kernel is asked for,
     // by name or by a launch geometry: both are bound by the binary64 pipe, and
     // the three passes issue fewer operations (no halo is evaluated twice).
-    // D2Q9 512^2, Nc = 4: fused 0.794 ms per step, three passes 0.261 ms.
+    // D2Q9 512^2, Nc = 4: fused 0.794 ms per step, three passes 0.260 ms.
     const bool prefer_fused = p->opt.precision != LBM_FP64 || p->opt.strip > 0 || p->opt.seg_h > 0;
     p->fused = can_fuse && (sched == LBM_SCHED_FUSED || (sched == LBM_SCHED_AUTO && prefer_fused));
     p->multipass = can_mp && (sched == LBM_SCHED_MULTIPASS || (sched == LBM_SCHED_AUTO && !p->fused));
     // LBM_FP32DEV on D2Q9: three node-parallel passes are faster than a row walk
     // while what they exchange (a population buffer, the new pairs and mu: 48 bytes
-    // per component and node) stays in L2; beyond, the fused kernel moves fewer
+    // per component, an odd number counted as the next, and node) stays in L2; beyond, the fused kernel moves fewer
     // bytes through DRAM.  Per step (graph), multi-pass / fused: 256^2 Nc = 3 11.9 /
     // 20.0 us, 512^2 Nc = 10 73 / 87 us, 1024^2 Nc = 2 69 / 71 us; past the line
     // 768^2 Nc = 6 102 / 95 us, 1024^2 Nc = 10 278 / 243 us.
@@ -754,9 +754,8 @@ int monitor_state(lbm_problem *p)
     return e;
 }
 
-// n steps of the resident schedule: launches of at most kResidentSteps steps (a
-// few milliseconds, so that other streams get their turn), ending where the
-// monitor reads the mass.  The state is advanced in place.
+// n steps of the resident schedule: launches of at most kResidentSteps steps (2.4 to 18
+// ms, on 16 of the SMs), ending where the monitor reads the mass.  The state is advanced in place.
 constexpr long long kResidentSteps = 1000;
 int resident_steps(lbm_problem *p, long long n)
 {

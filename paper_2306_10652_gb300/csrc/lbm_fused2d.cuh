@@ -623,7 +623,7 @@ __global__ void __launch_bounds__(kT, NC <= 10 && NC != 9 ? 4 : 3)
 // the components of a pair stored apart (twice the stores and addresses), 0.67 ms
 // with that and the inputs loaded into registers (spills, and every row waits for
 // its loads), 0.81 ms when it held the 80 populations of a node in registers,
-// component by component.  LBM_FP32 1021 x 1531, Nc = 6: 0.119 ms with four CTAs
+// component by component.  LBM_FP32 1021 x 1531, Nc = 6: 0.117 ms with four CTAs
 // per SM, 0.134 ms with three, 0.141 ms with three and the components apart, 0.260 ms
 // at first; Nc = 10 needs more than the 128 registers that four leave it.
 template <int NC, typename E, bool TAU1>

@@ -10,7 +10,7 @@
 // Both launches are bound by memory latency: the second summed all partials of a
 // component in one thread before, 85-115 us at any lattice size (128 x 4, Nc = 2:
 // 95 us for both, now 11), and the first had one CTA walk a chunk of every
-// component in turn (2048^2, Nc = 10, 335 MB: 312 us for both, now 217).
+// component in turn (2048^2, Nc = 10, 335 MB: 312 us for both, now 136).
 #include "lbm_internal.h"
 
 namespace lbmfug {

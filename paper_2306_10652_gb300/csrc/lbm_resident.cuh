@@ -19,8 +19,8 @@
 // Arithmetic by form: float (LBM_FP32), double (LBM_FP64), df::F2 (LBM_FP32DEV:
 // double-binary32 thermodynamics, binary32 collision, exact density pairs), with
 // the equations in the forms of the other kernels.
-// Per step: 400 x 2, Nc = 10, LBM_FP32 6.2 us (the fused kernel in a graph: 14.4 us),
-// LBM_FP32DEV 9.0 us (18.8 us); 128 x 4, Nc = 2, LBM_FP64 8.5 us (three passes:
+// Per step: 400 x 2, Nc = 10, LBM_FP32 6.6 us (the fused kernel in a graph: 14.4 us),
+// LBM_FP32DEV 8.7 us (18.8 us); 128 x 4, Nc = 2, LBM_FP64 8.6 us (three passes:
 // 16.9 us).  The floor, at a few hundred threads, is 2.4-3 us: three barriers and
 // the L2 round trips around them.
 #pragma once
@@ -81,7 +81,7 @@ template <int G> __device__ __forceinline__ float bfly_max(float v)
 
 // (binary32: the chain of a step hides most of logf, and __logf, whose absolute error is
 // 2^-21.4, is the largest rounding of mu: 400 x 2, Nc = 10, 200 steps, error of the
-// densities 5.3e-8 with logf, 1.1e-7 with __logf, at 6.4 and 6.2 us per step)
+// densities 5.3e-8 with logf, 1.1e-7 with __logf, at 6.6 and 6.3 us per step)
 __device__ __forceinline__ float lane_log(float x, const Log64 *) { return logf(x); }
 __device__ __forceinline__ double lane_log(double x, const Log64 *t) { return log64(x, t); }
 __device__ __forceinline__ float lane_rcp(float x) { return __fdividef(1.0f, x); }

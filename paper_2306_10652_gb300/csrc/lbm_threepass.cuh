@@ -17,8 +17,7 @@
 // binary64 operations and nothing else: one node per thread (no halo is
 // computed twice), mu formed once so that one gradient per component serves
 // the force, the collision evaluated as one quadratic form per component
-// (below), one reciprocal per node in the equation of state, and a
-// table-driven logarithm of 7 operations.
+// (below), reciprocals of 3 operations and a table-driven logarithm of 8.
 //
 // State formats (post-streaming populations, the convention of Eq. 1a):
 //  * binary64 (S = double): all Q populations g[i][a][node].
@@ -313,9 +312,9 @@ __global__ void __launch_bounds__(kThreads)
 // odd part and the two populations 2 each.  Written direction by direction the
 // same terms take about 20 operations per population, and the kernel is bound
 // by the binary64 pipe.  Whole step, with passes 1 and 2 as they stand now and
-// as they were: D2Q9 512^2, Nc = 4, 0.261 ms (the fused kernel that ran there:
-// 0.794 ms); D3Q19 51x47x45, Nc = 6, 0.286 ms (0.575 ms).  The pipe is 80-85 %
-// active in all three passes.
+// as they were: D2Q9 512^2, Nc = 4, 0.260 ms (the fused kernel that ran there:
+// 0.794 ms); D3Q19 51x47x45, Nc = 6, 0.290 ms (0.575 ms).  The pipe is 84 %
+// active in passes 2 and 3, 70 % in pass 1, which waits for its loads too.
 //
 // TAU1 (tau = 1, the paper's value): (1 - w) g_a vanishes, so the moving
 // populations are w g^eq + F/2 and the old ones are not read.
